@@ -264,11 +264,11 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-KERNEL_SOURCES = ("nr_device.cuh", "nr_mixed.cu", "nr_pair.cu")
+KERNEL_SOURCES = ("nr_device.cuh", "nr_pair.cuh", "nr_mixed.cu", "nr_pair.cu", "nr_roll.cu")
 
 
 def kernel_source_hash() -> str:
-    """Hash of the gradient kernels' sources (shared header, one- and
+    """Hash of the gradient kernels' sources (shared headers, one- and
     two-evaluations-per-thread kernels, in that order) with // comments and
     whitespace removed, so that an edit of the comments alone does not mark
     a capture of the same code as stale."""

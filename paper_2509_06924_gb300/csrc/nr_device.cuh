@@ -15,12 +15,13 @@
 namespace nrimpl {
 namespace {
 
-constexpr float kInv2Pi = 0.159154943091895335769f;
-constexpr float kTwoPiHi = 6.28318548202514648438f;      // float(2 pi)
-constexpr float kTwoPiLo = -1.74845553146951715e-07f;    // 2 pi - kTwoPiHi
 constexpr float kRoundMagic = 12582912.0f;               // 1.5 * 2^23: x + M - M rounds x to an integer
 constexpr double kFourPiD = 12.566370614359172953850573533118;
 constexpr double kLog2ED = 1.4426950408889634073599246810019; // log2(e)
+constexpr double kTwoStepsD = 40.743665431525205956834243423364; // 2 x 128 / (2 pi): d to 2 d in table steps
+// stacks whose Nevot-Croce phases all stay below this take sin / cos of them
+// from a polynomial without reduction (the paired kernels)
+constexpr float kNcSmall = 0.125f;
 constexpr float kLog2Pi = 1.83787706640934548356f;       // ln(2 pi)
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -75,8 +76,8 @@ __device__ __forceinline__ void sincos_approx(float x, float &sn, float &cs)
 // sin / cos of the layer phases and of the Nevot-Croce factors.
 // NR_SINCOS_TABLE 1: a 128-entry table of cos / sin at multiples of 2 pi / 128
 // (correctly rounded on the host, staged in shared memory) and two short
-// polynomials for the remainder |x| <= pi / 128 (sin: x - x^3 / 6, below
-// 1e-10; cos: 1 - c x^2 with c the minimax coefficient on that interval,
+// polynomials for the remainder |y| <= pi / 128 (sin: y - y^3 / 6, below
+// 1e-10; cos: 1 - c y^2 with c the minimax coefficient on that interval,
 // below 2.6e-9, where the Taylor c = 1/2 leaves a one-sided 1.5e-8),
 // combined by the angle-addition formula: about 1e-7 absolute, on the FMA
 // pipe plus one shared load.  0: the special-function unit's sin.approx /
@@ -95,29 +96,29 @@ __device__ __forceinline__ void sincos_approx(float x, float &sn, float &cs)
 
 constexpr int kTabN = kSinCosTabN;
 static_assert(kTabN == 128, "reduction constants are for 128 entries");
-constexpr float kTabScale = 20.3718318939209f;        // 128 / (2 pi)
-constexpr float kTabStepHi = 0.04908738657832146f;    // float(2 pi / 128)
-constexpr float kTabStepLo = -1.3659808839605603e-09f; // 2 pi / 128 - kTabStepHi
-// c of cos x ~ 1 - c x^2 minimising the largest error over |x| <= pi / 128
-constexpr float kTabCosC = 0.4999791979789734f;
+constexpr float kTabScale = 20.3718318939209f;   // 128 / (2 pi): radians to table steps
+constexpr float kTabStep = 0.04908738657832146f; // 2 pi / 128: table steps to radians
+// sin and 1 - cos of x table steps (|x| <= 1/2): x (kTabS1 + kTabS3 x^2) and
+// kTabC2 x^2, with c = 0.49997920 of 1 - c y^2 minimising the largest error over |y| <= pi / 128
+constexpr float kTabS1 = kTabStep;
+constexpr float kTabS3 = -1.9713260e-05f;        // -(2 pi / 128)^3 / 6
+constexpr float kTabC2 = -1.2047356e-03f;        // -c (2 pi / 128)^2
 
-// (cos, sin) of ph + pl (pl a low-order correction, |pl| << 1): reduction
-// by multiples of 2 pi / 128 (the multiple rounded with the 1.5 * 2^23
-// addition, whose low mantissa bits are then the table index), remainder
-// polynomials sin x ~ x - x^3 / 6, cos x ~ 1 - kTabCosC x^2.  tab: cos at
-// [i], sin at [kTabN + i].
+// (cos, sin) of the angle ph + pl given in table steps of 2 pi / 128 (pl a
+// low-order correction, |pl| << 1).  Staging the layer constants in steps
+// makes the reduction exact: the nearest integer (rounded with the
+// 1.5 * 2^23 addition, whose low mantissa bits are then the table index)
+// subtracts without error.  tab: cos at [i], sin at [kTabN + i].
 __device__ __forceinline__ float2 cis_tab(float ph, float pl, const float *tab)
 {
-    const float t = fmaf(ph, kTabScale, kRoundMagic);
+    const float t = __fadd_rn(ph, kRoundMagic);
     const float nt = __fadd_rn(t, -kRoundMagic);
     const int i = __float_as_int(t) & (kTabN - 1);
     const float2 cs = make_float2(tab[i], tab[kTabN + i]);
-    float x = fmaf(-nt, kTabStepHi, ph);
-    x = fmaf(-nt, kTabStepLo, x);
-    x = __fadd_rn(x, pl);
+    const float x = __fadd_rn(__fadd_rn(ph, -nt), pl);
     const float z = x * x;
-    const float sn = fmaf(x * z, -1.f / 6.f, x);
-    const float cn = fmaf(z, -kTabCosC, 1.f);
+    const float sn = x * fmaf(z, kTabS3, kTabS1);
+    const float cn = fmaf(z, kTabC2, 1.f);
     return make_float2(fmaf(cs.x, cn, -cs.y * sn), fmaf(cs.y, cn, cs.x * sn));
 }
 
@@ -237,10 +238,10 @@ __device__ __forceinline__ Kz medium_kz(float p_hi, float p_lo, float4 m)
     }
 }
 
-// E = exp(2 i k d).  The real phase 2 Re(k) d is formed in double-float and
-// reduced modulo 2 pi (Cody-Waite, two-word 2 pi; the multiple of 2 pi is
-// rounded with the 1.5 * 2^23 addition) before the FP32 sincos.
-// L = (2 d as (hi, lo), ea = -2 d log2(e), -): |E| = 2^(Im(k) ea).
+// E = exp(2 i k d).  The real phase 2 Re(k) d is formed in double-float, in
+// table steps of 2 pi / 128, and reduced by whole steps (or, for the
+// special-function unit, by whole turns) before the FP32 sin / cos.
+// L = (2 d in table steps as (hi, lo), ea = -2 d log2(e), -): |E| = 2^(Im(k) ea).
 __device__ __forceinline__ float2 layer_phase(const Kz &k, float4 L, const float *tab)
 {
     const float2 d2 = make_float2(L.x, L.y);
@@ -255,10 +256,8 @@ __device__ __forceinline__ float2 layer_phase(const Kz &k, float4 L, const float
     const float2 e = cis_tab(ph, pl, tab);
     return make_float2(amp * e.x, amp * e.y);
 #else
-    const float nt = __fadd_rn(fmaf(ph, kInv2Pi, kRoundMagic), -kRoundMagic);
-    float red = fmaf(-nt, kTwoPiHi, ph);
-    red = fmaf(-nt, kTwoPiLo, red);
-    red += pl;
+    const float nt = __fadd_rn(fmaf(ph, 1.f / kTabN, kRoundMagic), -kRoundMagic);
+    const float red = __fadd_rn(fmaf(-nt, (float)kTabN, ph), pl) * kTabStep;
     float s, c;
     sincos_approx(red, s, c);
     return make_float2(amp * c, amp * s);
@@ -285,7 +284,7 @@ __device__ __forceinline__ float2 fresnel_nc(float2 ka, float2 kb, float4 I, flo
     const float wi = s * kk.y;
     if (NR_BRANCHFREE || wi != 0.f) {
 #if NR_NC_TABLE
-        const float2 e = cis_tab(wi, 0.f, tab);
+        const float2 e = cis_tab(wi * kTabScale, 0.f, tab);
         F = make_float2(amp * e.x, amp * e.y);
 #else
         float sn, cs;
@@ -413,29 +412,30 @@ __device__ __forceinline__ void k0_square(float k0h, float k0l, float &p_hi, flo
 // Z and Xbar_{j-1}; k_{j-1}, k_j and k_{j+1} are formed again from the node
 // exactly as the sweeps form them.
 __device__ __forceinline__ float2 edge_entry_ubar(float2 node, float2 Z, float2 Xbu, int j, int n,
-                                                  const float4 *med, const float4 *lay)
+                                                  const float4 *med, const float4 *lay, const float4 *adj)
 {
     float p_hi, p_lo;
     k0_square(node.x, node.y, p_hi, p_lo);
     const Kz ka = j == 1 ? Kz{node.x, 0.f, node.y} : medium_kz<true>(p_hi, p_lo, med[j - 1]);
     const Kz kj = medium_kz<true>(p_hi, p_lo, med[j]);
     const Kz kb = j == n ? medium_kz<false>(p_hi, p_lo, med[j + 1]) : medium_kz<true>(p_hi, p_lo, med[j + 1]);
-    return edge_ubar(kc(ka), kc(kj), kc(kb), lay[j - 1].w, lay[j].w, 0.5f * lay[j].x, Z, j == n, Xbu);
+    return edge_ubar(kc(ka), kc(kj), kc(kb), lay[j - 1].w, lay[j].w, 0.5f * adj[j - 1].w, Z, j == n, Xbu);
 }
 
 // Drains `cnt` queued interior-edge entries of one warp (one per lane) into
 // per-thread partials kept in shared memory (acc points at this thread's
 // slot of medium 1's Re-accumulator; stride between accumulators `stride`,
-// Re -> Im distance `im_off`; med, lay: the staged stack entries).  Kept out
+// Re -> Im distance `im_off`; med, lay, adj: the staged stack entries).  Kept out
 // of line so that the rolled sweep it is called from keeps its register budget.
 template <int EQ, bool RES>
 __device__ __noinline__ float eq_drain_smem(float2 (*q)[EQ], const int *qj, const float4 *med, const float4 *lay,
-                                            int n, int lane, int cnt, float *acc, int stride, int im_off)
+                                            const float4 *adj, int n, int lane, int cnt, float *acc, int stride,
+                                            int im_off)
 {
     float res = 0.f; // the resolution-mode term of the entry (factor in q[3])
     if (lane < cnt) {
         const int j = qj[lane];
-        const float2 ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, lay);
+        const float2 ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, lay, adj);
         // conj(kbar)/k_j = 2 conj(ubar)
         acc[(j - 1) * stride] += 2.f * ub.x;
         acc[(j - 1) * stride + im_off] += -2.f * ub.y;
@@ -472,8 +472,12 @@ struct StackSmem {
     float4 med[NM + 2]; // medium j = 1..n+1: 4 pi (rho_j - rho_0) as (hi, lo), 4 pi iota_j, its square
     float4 itf[NM + 1]; // interface j = 0..n: 4 pi (rho_{j+1} - rho_j) + 4 pi i (iota_j - iota_{j+1}),
                         // s_j = -2 sigma_j^2, s_j log2(e)
-    float4 lay[NM + 2]; // layer j = 1..n: 2 d_j as (hi, lo), -2 d_j log2(e); sigma_j (j = 0..n)
+    float4 lay[NM + 2]; // layer j = 1..n: 2 d_j in table steps (x 128 / 2 pi) as (hi, lo), -2 d_j log2(e);
+                        // sigma_j (j = 0..n)
+    float4 adj[NM + 1]; // interface j = 0..n: the adjoint's constants Re(s_j conj(N_j)) + 2 and - 2,
+                        // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
     float scale, bkg;
+    int nc_big;         // 1: some interface's Nevot-Croce phase may exceed kNcSmall (cleared by the item's owner)
 };
 
 __device__ __forceinline__ float2 split_double(double v)
@@ -499,7 +503,7 @@ __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, 
             bad |= !isfinite(rj) || !isfinite(ij);
             if (j <= n) {
                 const double dj = p[j - 1];
-                const float2 d2 = split_double(2.0 * dj);
+                const float2 d2 = split_double(dj * kTwoStepsD);
                 lay.x = d2.x;
                 lay.y = d2.y;
                 lay.z = (float)(-2.0 * kLog2ED * dj);
@@ -512,11 +516,21 @@ __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, 
             const double iot_j = j >= 1 ? p[2 * n + 2 + j - 1] : 0.0;
             const double iot_j1 = p[2 * n + 2 + j];
             const double sig = p[3 * n + 3 + j];
-            sm.itf[j] = make_float4((float)(kFourPiD * (p[n + j + 1] - p[n + j])),
-                                    (float)(kFourPiD * (iot_j - iot_j1)), (float)(-2.0 * sig * sig),
-                                    (float)(-2.0 * kLog2ED * sig * sig));
+            const float Nr = (float)(kFourPiD * (p[n + j + 1] - p[n + j]));
+            const float Ni = (float)(kFourPiD * (iot_j - iot_j1));
+            const float s = (float)(-2.0 * sig * sig);
+            sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig * sig));
+            sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, j < n ? (float)(2.0 * p[j]) : 0.f);
             lay.w = (float)sig;
             bad |= !isfinite(sig);
+            // |s Im(k_j k_{j+1})| <= -s (D / 2 + sqrt(5 m a) + a) with
+            // D = |Re N|, a the larger 4 pi iota of the two media, m = max(D, a):
+            // with k^2 = u + i a of each, 2 Im^2 = |z z'| - Re(z z') is at most
+            // D^2 / 2 where u and u' differ in sign, plus |u| a' + |u'| a
+            // + 2 a a'; for |u| > 4 m of one sign it is below (0.6 (a + a'))^2 x 2
+            const float D = fabsf(Nr), a = (float)kFourPiD * fmaxf(fabsf((float)iot_j), fabsf((float)iot_j1));
+            const float bound = -s * (0.5f * D + sqrtf(5.f * fmaxf(D, a) * a) + 1.2f * a);
+            if (!(bound <= kNcSmall)) sm.nc_big = 1; // every writer stores the same value
         }
         sm.lay[j] = lay;
         if (j == 0) {

@@ -126,13 +126,18 @@ cudaError_t launch_mixed(int mode, int nmax, int grid, const KernelArgs &a, cons
 bool mixed_bucket_ok(int mode, int nmax);
 
 // ---- paired kernel (nr_pair.cu): two evaluations per thread ----
-// Used by launch_mixed / mixed_occupancy / mixed_tile_q when K >= 3 for the
-// 1- and 2-layer gradient buckets and the 1-layer forward (model, loglik)
-// bucket.
+// Used by launch_mixed / mixed_occupancy / mixed_tile_q when K >= 3, for every
+// bucket (gradients of more than two layers: nr_roll.cu, below).
 bool pair_eligible(int mode, int nmax, int K);
 int pair_block_threads();
 cudaError_t pair_occupancy(int mode, int nmax, int K, int *blocks_per_sm);
 cudaError_t launch_pair(int mode, int nmax, int grid, const KernelArgs &a, const QuadConst &qc, cudaStream_t st);
+
+// ---- gradient kernels of 3 to 64 layers (nr_roll.cu), reached through the two above ----
+// One CTA per SM holds several teams, each a consumer of the work queue:
+// "occupancy" and the launch's size count teams.
+cudaError_t roll_occupancy(int mode, int nmax, int *teams_per_sm);
+cudaError_t launch_roll(int mode, int nmax, int workers, const KernelArgs &a, const QuadConst &qc, cudaStream_t st);
 
 // ---- launchers (nr_fp64.cu) ----
 constexpr int kFp64Block = 128;

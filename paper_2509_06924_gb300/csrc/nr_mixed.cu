@@ -1,9 +1,8 @@
 // nr_mixed.cu -- batched reflectivity, log-likelihood and its exact gradient
 // in complex FP32 with double-float guards, for sm_103a, one evaluation per
-// thread.  The two-evaluations-per-thread kernels of nr_pair.cu run instead
-// wherever they apply (K >= 3, gradient buckets up to 20 layers, both forward
-// buckets); this kernel serves K < 3, the 32- and 64-layer gradient buckets,
-// and builds with NR_PAIR=0, and the autotuner may pick it per bucket.
+// thread.  The two-evaluations-per-thread kernels (nr_pair.cu, nr_roll.cu) run
+// instead wherever they apply (K >= 3); this kernel serves K < 3 and builds
+// with NR_PAIR=0, and the autotuner may pick it per bucket.
 //
 // Work decomposition.  A work item is a range of Q points of one stack.  A
 // persistent CTA takes items from a queue (atomic ticket, cost-sorted on the
@@ -241,12 +240,12 @@ nr_mixed_kernel(const KernelArgs ka, const QuadConst qc)
         // drain `cnt` <= 32 queued entries, one per lane, then shift the rest down
         auto eq_drain = [&](int cnt) {
             if constexpr (T::SMEM_ACC) {
-                gres_acc += eq_drain_smem<EQ, RES>(sh_eq[warp], sh_eqj[warp], sm.med, sm.lay, n, lane, cnt,
-                                                   sh_acc + oUr * BLOCK + tid, BLOCK, (oUi - oUr) * BLOCK);
+                gres_acc += eq_drain_smem<EQ, RES>(sh_eq[warp], sh_eqj[warp], sm.med, sm.lay, sm.adj, n, lane,
+                                                   cnt, sh_acc + oUr * BLOCK + tid, BLOCK, (oUi - oUr) * BLOCK);
             } else if (lane < cnt) {
                 const int j = sh_eqj[warp][lane];
                 const float2 ub = edge_ubar(sh_eq[warp][0][lane], sh_eq[warp][1][lane], sh_eq[warp][2][lane],
-                                            sm.lay[j - 1].w, sm.lay[j].w, 0.5f * sm.lay[j].x, sh_eq[warp][3][lane],
+                                            sm.lay[j - 1].w, sm.lay[j].w, 0.5f * sm.adj[j - 1].w, sh_eq[warp][3][lane],
                                             j == n, sh_eq[warp][4][lane]);
                 // conj(kbar)/k_j = 2 conj(ubar)
                 acc_u(j, make_float2(2.f * ub.x, -2.f * ub.y));
@@ -494,7 +493,7 @@ nr_mixed_kernel(const KernelArgs ka, const QuadConst qc)
                 auto adj_step = [&](int j, auto TOP, auto BOT, auto EDG) __attribute__((always_inline)) {
                     const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                     const float4 Ij = sm.itf[j];
-                    const float4 Lj1 = sm.lay[j + 1]; // layer j+1 (zeros past the last layer)
+                    [[maybe_unused]] const float4 Lj1 = sm.lay[j + 1]; // layer j+1 (zeros past the last layer)
                     const float2 Xb_in = Xb;
                     float2 Zj = make_float2(0.f, 0.f);
                     Kz kj1;
@@ -538,7 +537,7 @@ nr_mixed_kernel(const KernelArgs ka, const QuadConst qc)
                         // Re(k) Im(U) - Im(k) Re(U) (halved) and kbar_{j+1} = -2 i d U.
                         const float2 U = cmulc(Y, Yb);
                         acc_fma2(oD + j, kj1.re, U.y, -kj1.im, U.x);
-                        const float dd = Lj1.x;
+                        const float dd = sm.adj[j].w;
                         kbar1 = make_float2(dd * U.y, -dd * U.x);
                     } else {
                         rb = Xb;

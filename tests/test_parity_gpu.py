@@ -323,6 +323,43 @@ def test_paired_gradient_kernel_orders_and_buckets(K):
     assert res_err(wl, g, gr, ref_g, ref_r) <= TOL_G
 
 
+# Gradients of more than two layers keep their factors in tensor memory, with
+# a different number of teams per SM and columns per thread from bucket to
+# bucket (edges at 4, 8, 12, 16, 20, 32, 64 layers).  Beside random stacks:
+# adjoining equal media without roughness (r = 0), and roughnesses whose
+# Nevot-Croce phase needs the reduced sin / cos instead of the polynomial.
+# The bounds are the module's, which hold at every depth.
+@pytest.mark.parametrize("K", [3, 17, 21, 32])
+def test_rolled_gradient_kernel_bucket_edges(K):
+    rng = np.random.default_rng(300 + K)
+    q1, q2 = W.log_grid(53, 0.005, 0.25), W.log_grid(23, 0.008, 0.03)
+    datasets = [(q1, 0.04 * q1), (q2, 0.05 * q2)]
+    stacks = [(n, rand_stack(rng, n, d_range=(5, 60)) if n > 20 else rand_stack(rng, n), n % 2)
+              for n in (3, 4, 5, 8, 9, 12, 13, 16, 17, 20, 21, 32, 33, 64)]
+    rho = [0.0, 4e-6, 4e-6, 4e-6, 1e-6, 2.07e-6]
+    stacks.append((4, W.pack([120.0, 80.0, 0.0, 200.0], rho, np.zeros(5), [4.0, 0.0, 0.0, 3.0, 0.0], 1.0, 1e-7), 0))
+    for n in (3, 7, 14):
+        st = rand_stack(rng, n, d_range=(200, 600))
+        L = W.layout(n)
+        st[L["sigma"]] = rng.uniform(40, 80, n + 1)
+        stacks.append((n, st, n % 2))
+    wl = custom_workload(stacks, datasets, K=K)
+    ref_ll, ref_g, ref_r = oracle.batch("grad_res", wl.n_layers, wl.params, wl.dataset, wl.q_off, wl.q, wl.dq,
+                                        wl.r_obs, wl.r_err, K)
+    ref = {"ll": ref_ll, "g": ref_g, "m": run_oracle(wl, modes=("model",))["m"]}
+    assert_parity(wl, run_gpu(wl), ref)
+    # several items per stack, more teams than items, and the resolution derivative
+    ctx = nr.Context(n_quad=K, chunk_q=9, tile_q=5)
+    ll, g, gr = (t.cpu().numpy() for t in ctx.loglik_grad_res(nr.Batch.from_workload(wl)))
+    assert ctx.device_status() == 0
+    ctx.close()
+    po = wl.par_off
+    e_res = [res_err(wl.subset([i]), g[po[i]:po[i + 1]], gr[i:i + 1], ref_g[po[i]:po[i + 1]], ref_r[i:i + 1])
+             for i in range(wl.n_stacks)]
+    check_bounds(wl, {"loglik": np.abs(ll - ref_ll) / np.abs(ref_ll), "grad": np.array(e_res)},
+                 {"loglik": TOL_LL, "grad": TOL_G})
+
+
 def test_zero_resolution_is_unsmeared():
     wl = W.make_workload("thick_oxide", n_stacks=16)
     wl.dq = np.zeros_like(wl.dq)
