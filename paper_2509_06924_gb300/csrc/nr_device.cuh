@@ -412,30 +412,30 @@ __device__ __forceinline__ void k0_square(float k0h, float k0l, float &p_hi, flo
 // Z and Xbar_{j-1}; k_{j-1}, k_j and k_{j+1} are formed again from the node
 // exactly as the sweeps form them.
 __device__ __forceinline__ float2 edge_entry_ubar(float2 node, float2 Z, float2 Xbu, int j, int n,
-                                                  const float4 *med, const float4 *lay, const float4 *adj)
+                                                  const float4 *med, const float *sig, const float4 *adj)
 {
     float p_hi, p_lo;
     k0_square(node.x, node.y, p_hi, p_lo);
     const Kz ka = j == 1 ? Kz{node.x, 0.f, node.y} : medium_kz<true>(p_hi, p_lo, med[j - 1]);
     const Kz kj = medium_kz<true>(p_hi, p_lo, med[j]);
     const Kz kb = j == n ? medium_kz<false>(p_hi, p_lo, med[j + 1]) : medium_kz<true>(p_hi, p_lo, med[j + 1]);
-    return edge_ubar(kc(ka), kc(kj), kc(kb), lay[j - 1].w, lay[j].w, 0.5f * adj[j - 1].w, Z, j == n, Xbu);
+    return edge_ubar(kc(ka), kc(kj), kc(kb), sig[j - 1], sig[j], 0.5f * adj[j - 1].w, Z, j == n, Xbu);
 }
 
 // Drains `cnt` queued interior-edge entries of one warp (one per lane) into
 // per-thread partials kept in shared memory (acc points at this thread's
 // slot of medium 1's Re-accumulator; stride between accumulators `stride`,
-// Re -> Im distance `im_off`; med, lay, adj: the staged stack entries).  Kept out
+// Re -> Im distance `im_off`; med, sig, adj: the staged stack entries).  Kept out
 // of line so that the rolled sweep it is called from keeps its register budget.
 template <int EQ, bool RES>
-__device__ __noinline__ float eq_drain_smem(float2 (*q)[EQ], const int *qj, const float4 *med, const float4 *lay,
+__device__ __noinline__ float eq_drain_smem(float2 (*q)[EQ], const int *qj, const float4 *med, const float *sig,
                                             const float4 *adj, int n, int lane, int cnt, float *acc, int stride,
                                             int im_off)
 {
     float res = 0.f; // the resolution-mode term of the entry (factor in q[3])
     if (lane < cnt) {
         const int j = qj[lane];
-        const float2 ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, lay, adj);
+        const float2 ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, sig, adj);
         // conj(kbar)/k_j = 2 conj(ubar)
         acc[(j - 1) * stride] += 2.f * ub.x;
         acc[(j - 1) * stride + im_off] += -2.f * ub.y;
@@ -473,7 +473,8 @@ struct StackSmem {
     float4 itf[NM + 1]; // interface j = 0..n: 4 pi (rho_{j+1} - rho_j) + 4 pi i (iota_j - iota_{j+1}),
                         // s_j = -2 sigma_j^2, s_j log2(e)
     float4 lay[NM + 2]; // layer j = 1..n: 2 d_j in table steps (x 128 / 2 pi) as (hi, lo), -2 d_j log2(e);
-                        // sigma_j (j = 0..n)
+                        // 4 pi (iota_{j-1} + iota_j) of the media above and in it (j = 1..n+1)
+    float sig[NM + 1];  // sigma_j, j = 0..n
     float4 adj[NM + 1]; // interface j = 0..n: the adjoint's constants Re(s_j conj(N_j)) + 2 and - 2,
                         // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
     float scale, bkg;
@@ -500,6 +501,7 @@ __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, 
             const double ij = p[2 * n + 2 + j - 1];
             const float2 c = split_double(kFourPiD * (rj - rho0));
             sm.med[j] = make_float4(c.x, c.y, (float)(kFourPiD * ij), (float)(kFourPiD * kFourPiD * ij * ij));
+            lay.w = (float)(kFourPiD * (ij + (j >= 2 ? p[2 * n + 2 + j - 2] : 0.0)));
             bad |= !isfinite(rj) || !isfinite(ij);
             if (j <= n) {
                 const double dj = p[j - 1];
@@ -521,7 +523,7 @@ __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, 
             const float s = (float)(-2.0 * sig * sig);
             sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig * sig));
             sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, j < n ? (float)(2.0 * p[j]) : 0.f);
-            lay.w = (float)sig;
+            sm.sig[j] = (float)sig;
             bad |= !isfinite(sig);
             // |s Im(k_j k_{j+1})| <= -s (D / 2 + sqrt(5 m a) + a) with
             // D = |Re N|, a the larger 4 pi iota of the two media, m = max(D, a):

@@ -240,12 +240,12 @@ nr_mixed_kernel(const KernelArgs ka, const QuadConst qc)
         // drain `cnt` <= 32 queued entries, one per lane, then shift the rest down
         auto eq_drain = [&](int cnt) {
             if constexpr (T::SMEM_ACC) {
-                gres_acc += eq_drain_smem<EQ, RES>(sh_eq[warp], sh_eqj[warp], sm.med, sm.lay, sm.adj, n, lane,
+                gres_acc += eq_drain_smem<EQ, RES>(sh_eq[warp], sh_eqj[warp], sm.med, sm.sig, sm.adj, n, lane,
                                                    cnt, sh_acc + oUr * BLOCK + tid, BLOCK, (oUi - oUr) * BLOCK);
             } else if (lane < cnt) {
                 const int j = sh_eqj[warp][lane];
                 const float2 ub = edge_ubar(sh_eq[warp][0][lane], sh_eq[warp][1][lane], sh_eq[warp][2][lane],
-                                            sm.lay[j - 1].w, sm.lay[j].w, 0.5f * sm.adj[j - 1].w, sh_eq[warp][3][lane],
+                                            sm.sig[j - 1], sm.sig[j], 0.5f * sm.adj[j - 1].w, sh_eq[warp][3][lane],
                                             j == n, sh_eq[warp][4][lane]);
                 // conj(kbar)/k_j = 2 conj(ubar)
                 acc_u(j, make_float2(2.f * ub.x, -2.f * ub.y));

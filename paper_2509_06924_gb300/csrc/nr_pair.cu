@@ -13,13 +13,13 @@
 // both halves (free on the hardware), negated operands are free as well;
 // nothing is swapped between the halves, which would cost moves.
 //
-// The recursion runs in projective form (nr_pair.cuh); with Nevot-Croce
-// phases by polynomial where the stack's roughnesses allow it and layer
-// phases staged in table steps that took, against the Moebius form:
-// 16384 one-layer stacks x 400 Q x 21 nodes, gradient 1.464 -> 1.386 ms,
-// log-likelihood 0.820 -> 0.810 ms; 12288 ten-layer stacks, model curves
-// 1.779 -> 1.548 ms; 10000 stacks of 1-20 layers, log-likelihood 1.623 ->
-// 1.522 ms.
+// The recursion runs in projective form (nr_pair.cuh), Nevot-Croce phases come
+// from a polynomial where the stack's roughnesses allow it, layer phases are
+// staged in table steps, and the Fresnel factor takes S^2 from the media's
+// known k^2.  Against the Moebius form with table phases: 16384 one-layer
+// stacks x 400 Q x 21 nodes, gradient 1.464 -> 1.340 ms, log-likelihood 0.820
+// -> 0.802 ms; 12288 ten-layer stacks, model curves 1.779 -> 1.466 ms; 10000
+// stacks of 1-20 layers, log-likelihood 1.623 -> 1.512 ms.
 //
 // The forward modes run the same code up to the smearing sum (model: write
 // scale S + bkg; log-likelihood: the residual terms) and no adjoint.
@@ -195,7 +195,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             if (lane < cnt) {
                 const int j = sh_eqj[warp][lane];
                 const float2 ub = edge_ubar(sh_eq[warp][0][lane], sh_eq[warp][1][lane], sh_eq[warp][2][lane],
-                                            sm.lay[j - 1].w, sm.lay[j].w, 0.5f * sm.adj[j - 1].w, sh_eq[warp][3][lane],
+                                            sm.sig[j - 1], sm.sig[j], 0.5f * sm.adj[j - 1].w, sh_eq[warp][3][lane],
                                             j == n, sh_eq[warp][4][lane]);
                 // conj(kbar)/k_j = 2 conj(ubar)
 #pragma unroll
@@ -321,11 +321,11 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             auto fwd_step = [&](int j, auto TOP, auto BOT, auto TRIG) __attribute__((always_inline)) {
                 const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                 Kz2 kj;
-                if (top) kj = Kz2{k0h, bc(0.f), k0l};
+                if (top) kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
                 else kj = medium_kz2<true>(p_hi, p_lo, sm.med[j]);
                 const float4 Ij = sm.itf[j];
-                const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kc2(kj), kc2(kbelow), Ij, sh_cs)
-                                  : fresnel_g2<false, decltype(TRIG)::value>(kc2(kj), kc2(kbelow), Ij, sh_cs);
+                const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs)
+                                  : fresnel_g2<false, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs);
                 const c2 rj = cscl2(Ij.x, Ij.y, Gj);
                 if (bot) {
                     B = rj;
@@ -444,7 +444,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     const f2 mR = pneg(pmul(Rb2, R));
                     c2 Ab = c2{pmul(iA.re, mR), pneg(pmul(iA.im, mR))};
                     c2 kbar = czero();
-                    Kz2 kj = Kz2{k0h, bc(0.f), k0l};
+                    Kz2 kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
                     c2 Xb_up = czero(); // Xbar_{j-1} (edge sweeps)
                     Kz2 kjm1 = kj;
                     const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
@@ -487,10 +487,10 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                             kbar = cscla2(Cj.x, Cj.z, ga, kbar);
                             // k_j complete: accumulate conj(kbar) / k_j, or queue the
                             // interior-edge evaluation
-                            const f2 m2 = pfma(kj.re, kj.re, pmul(kj.im, kj.im));
                             b2 edge{false, false};
                             if constexpr (decltype(EDG)::value) {
-                                edge = b2{act[0] && m2.x < edge_u.x, act[1] && m2.y < edge_u.y};
+                                const f2 far = pmul(edge_u, kj.y); // |k_j|^2 < edge_u
+                                edge = b2{act[0] && far.x > 1.f, act[1] && far.y > 1.f};
 #pragma unroll
                                 for (int h = 0; h < 2; ++h) {
                                     const bool eh = h ? edge.y : edge.x;
@@ -518,7 +518,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                                 }
                             }
                             const c2 kq = cmul2(kbar, kc2(kj));
-                            f2 inv = prcp(pmax(m2, bc(1e-30f)));
+                            f2 inv = kj.y;
                             if constexpr (decltype(EDG)::value) inv = psel(edge, bc(0.f), inv);
                             const f2 ur = pmul(kq.re, inv);
                             accr[oUr + j - 1] = padd(accr[oUr + j - 1], ur);
@@ -531,8 +531,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                         kj = kj1;
                         if (bot) { // backing medium n+1
                             const c2 kk = cmul2(kbar, kc2(kj));
-                            const f2 m2 = pfma(kj.re, kj.re, pmul(kj.im, kj.im));
-                            const f2 inv = prcp(pmax(m2, bc(1e-30f)));
+                            const f2 inv = kj.y;
                             const f2 ur = pmul(kk.re, inv);
                             accr[oUr + j] = padd(accr[oUr + j], ur);
                             accr[oUi + j] = pfma(pneg(kk.im), inv, accr[oUi + j]);

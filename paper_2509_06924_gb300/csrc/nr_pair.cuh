@@ -48,14 +48,14 @@ __device__ __forceinline__ void pcis_tab(f2 ph, f2 pl, const float *tab, f2 &cs,
     cs = pfma(tc, cx, pneg(pmul(ts, sx)));
     sn = pfma(ts, cx, pmul(tc, sx));
 }
-// (cos, sin) of |x| <= kNcSmall radians without reduction: Taylor, truncation
-// below 6e-9 (cos) and 1e-10 (sin), six operations against the table's
-// twelve and its four shared loads
+// (cos, sin) of |x| <= kNcSmall = 1/8 radians without reduction: minimax
+// x (1 - d + b x^2) and 1 + x^2 (c + e x^2), within 1.6e-8 and 2e-10; five
+// operations against the table's twelve and its four shared loads
 __device__ __forceinline__ void pcis_small(f2 x, f2 &cs, f2 &sn)
 {
     const f2 z = pmul(x, x);
-    cs = pfma(z, pfma(z, bc(1.f / 24.f), bc(-0.5f)), bc(1.f));
-    sn = pfma(pmul(x, z), pfma(z, bc(1.f / 120.f), bc(-1.f / 6.f)), x);
+    cs = pfma(z, pfma(z, bc(0.04163646f), bc(-0.49999985f)), bc(1.f));
+    sn = pmul(x, pfma(z, bc(-0.16650396f), bc(0.99999936f)));
 }
 
 // error-free transformations on both halves (every paired add rounds once)
@@ -101,9 +101,10 @@ __device__ __forceinline__ c2 cfmac2(c2 a, c2 b, c2 c)
     return c2{pfma(a.re, b.re, pfma(a.im, b.im, c.re)), pfma(a.re, b.im, pfma(pneg(a.im), b.re, c.im))};
 }
 
-// wavevector of both evaluations (value + low word of Re k, as Kz)
+// wavevector of both evaluations (value + low word of Re k, as Kz), its
+// square's real part u and 1 / |k|^2, by-products of the root
 struct Kz2 {
-    f2 re, im, lo;
+    f2 re, im, lo, u, y;
 };
 __device__ __forceinline__ c2 kc2(const Kz2 &k) { return c2{k.re, k.im}; }
 
@@ -112,15 +113,16 @@ __device__ __forceinline__ c2 kc2(const Kz2 &k) { return c2{k.re, k.im}; }
 template <bool REFINE>
 __device__ __forceinline__ Kz2 kz_sqrt2(f2 uh, f2 ul, float a, float a2)
 {
+    Kz2 k;
+    k.u = uh;
     const f2 au = pabs(uh);
     const f2 m2 = pfma(uh, uh, bc(a2));
-    const f2 m = pmul(m2, prsqrt(pmax(m2, bc(1e-37f))));
-    const f2 H = padd(au, m);                             // |u| + |z| = 2 t^2
-    const f2 i2t = prsqrt(pmax(padd(H, H), bc(4e-30f))); // 1 / (2 t)
+    k.y = prsqrt(pmax(m2, bc(1e-37f)));
+    const f2 H = pfma(m2, k.y, au);                          // |u| + |z| = 2 t^2
+    const f2 i2t = prsqrt(pfma(H, bc(2.f), bc(4e-30f)));     // 1 / (2 t)
     const f2 t = pmul(H, i2t);
     const f2 small = pmul(bc(a), i2t);
     const b2 prop{uh.x >= 0.f, uh.y >= 0.f};
-    Kz2 k;
     if constexpr (REFINE) {
         const f2 e = padd(pfma(pneg(t), t, au), pfma(small, small, psel(prop, ul, pneg(ul))));
         const f2 corr = pmul(e, i2t);
@@ -176,21 +178,20 @@ __device__ __forceinline__ c2 layer_phase2(const Kz2 &k, float4 L, const float *
     return c2{pmul(amp, c), pmul(amp, s)};
 }
 
-// G = exp(s k_a k_b) / (k_a + k_b)^2, the Nevot-Croce Fresnel coefficient
-// without its numerator: r = N G.  With S = k_a + k_b and w = exp(s Re) / |S|^4,
-// G = w (cos + i sin) conj(S^2).  REAL_A: k_a is real (the fronting medium).
-// A vanishing S (k_a = k_b = 0) gives a finite G whose numerator is 0.
+// G = exp(s k_a k_b) / S^2, S = k_a + k_b: the Nevot-Croce Fresnel
+// coefficient without its numerator, r = N G.  S^2 = k_a^2 + k_b^2 + 2 k_a k_b
+// takes the squares as they are known (u_a + u_b + i aa, aa the sum of both
+// media's 4 pi iota), and G = w (cos + i sin) conj(S^2) with w = exp(s Re) /
+// |S^2|^2.  REAL_A: k_a is real (the fronting medium).  A vanishing S
+// (k_a = k_b = 0) gives a finite G whose numerator is 0.
 template <bool REAL_A, int TRIG>
-__device__ __forceinline__ c2 fresnel_g2(c2 ka, c2 kb, float4 I, const float *tab)
+__device__ __forceinline__ c2 fresnel_g2(const Kz2 &ka, const Kz2 &kb, float4 I, float aa, const float *tab)
 {
-    const f2 Sx = padd(ka.re, kb.re);
-    const f2 Sy = REAL_A ? kb.im : padd(ka.im, kb.im);
-    const f2 sy2 = pmul(Sy, Sy);
-    const f2 inv = prcp(pmax(pfma(Sx, Sx, sy2), bc(1e-18f)));
-    const f2 A = pfma(Sx, Sx, pneg(sy2));         // Re S^2
-    const f2 B = pmul(padd(Sx, Sx), Sy);          // Im S^2
-    const c2 kk = REAL_A ? c2{pmul(ka.re, kb.re), pmul(ka.re, kb.im)} : cmul2(ka, kb);
-    const f2 w = pmul(pmul(pex2(pmul(bc(I.w), kk.re)), inv), inv);
+    const c2 kk = REAL_A ? c2{pmul(ka.re, kb.re), pmul(ka.re, kb.im)} : cmul2(kc2(ka), kc2(kb));
+    const f2 A = pfma(bc(2.f), kk.re, padd(ka.u, kb.u)); // Re S^2
+    const f2 B = pfma(bc(2.f), kk.im, bc(aa));           // Im S^2
+    const f2 inv = prcp(pmax(pfma(A, A, pmul(B, B)), bc(1e-36f)));
+    const f2 w = pmul(pex2(pmul(bc(I.w), kk.re)), inv);
     const f2 ph = pmul(bc(I.z), kk.im);
     f2 sn, cs;
     if constexpr (TRIG == kTrigSmall) pcis_small(ph, cs, sn);

@@ -125,7 +125,7 @@ __device__ __forceinline__ void team_sync(int team)
 // order of the additions is fixed.  Kept out of line (rare).
 template <bool RES>
 __device__ __noinline__ float roll_drain(const float2 (*q)[kEqCap], const int *qj, const float *qr, const float4 *med,
-                                         const float4 *lay, const float4 *adj, int n, int lane, int cnt, float *acc)
+                                         const float *sig, const float4 *adj, int n, int lane, int cnt, float *acc)
 {
     float res = 0.f;
     const bool on = lane < cnt;
@@ -134,7 +134,7 @@ __device__ __noinline__ float roll_drain(const float2 (*q)[kEqCap], const int *q
     __syncwarp();
     if (on) {
         j = qj[lane];
-        ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, lay, adj);
+        ub = edge_entry_ubar(q[0][lane], q[1][lane], q[2][lane], j, n, med, sig, adj);
         if constexpr (RES) res = 2.f * ub.x * qr[lane];
     }
     for (int turn = 0; turn < 4; ++turn) {
@@ -250,7 +250,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         f2 gres_acc = bc(0.f);
         int eq_cnt = 0; // entries in this warp's interior-edge queue (warp-uniform)
         auto eq_drain = [&]() {
-            const float r = roll_drain<RES>(ts.eq[warp], ts.eqj[warp], RES ? ts.eqr[warp] : nullptr, sm.med, sm.lay,
+            const float r = roll_drain<RES>(ts.eq[warp], ts.eqj[warp], RES ? ts.eqr[warp] : nullptr, sm.med, sm.sig,
                                             sm.adj, n, lane, eq_cnt, acc);
             if constexpr (RES) gres_acc.x += r;
             eq_cnt = 0;
@@ -352,7 +352,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 {
                     const Kz2 kj = medium_kz2<true>(p_hi, p_lo, sm.med[n]);
                     const float4 I = sm.itf[n];
-                    const c2 G = fresnel_g2<false, T>(kc2(kj), kc2(kb), I, sh_cs);
+                    const c2 G = fresnel_g2<false, T>(kj, kb, I, sm.lay[n + 1].w, sh_cs);
                     B = cscl2(I.x, I.y, G);
                     ts.b[NM * kTeam + tid] = make_float4(G.re.x, G.re.y, G.im.x, G.im.y);
                     kb = kj;
@@ -360,11 +360,12 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 auto step = [&](int j, auto TOP) __attribute__((always_inline)) {
                     constexpr bool top = decltype(TOP)::value;
                     Kz2 kj;
-                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l};
+                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
                     else kj = medium_kz2<true>(p_hi, p_lo, sm.med[j]);
                     const float4 I = sm.itf[j];
-                    const c2 G = fresnel_g2<top, T>(kc2(kj), kc2(kb), I, sh_cs);
-                    const c2 E = layer_phase2<true>(kb, sm.lay[j + 1], sh_cs);
+                    const float4 L = sm.lay[j + 1];
+                    const c2 G = fresnel_g2<top, T>(kj, kb, I, L.w, sh_cs);
+                    const c2 E = layer_phase2<true>(kb, L, sh_cs);
                     tmem_store(tm + j * kSlotCols, G, E);
                     const c2 r = cscl2(I.x, I.y, G);
                     const c2 b = cmul2(B, E);
@@ -426,6 +427,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             c2 Ab = c2{pmul(iA.re, mR), pneg(pmul(iA.im, mR))};
             c2 kbar = czero();
             c2 kj = c2{k0h, bc(0.f)};
+            f2 yj = bc(0.f); // 1 / |k_j|^2
             c2 Xb_up = czero(); // Xbar_{j-1} (edge sweeps)
             const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
             const f2 wres = RES ? pmul(dQh, g_hi) : bc(0.f);
@@ -437,7 +439,8 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 Slot sl;
                 if constexpr (!bot) tmem_load(tm + j * kSlotCols, sl);
                 const float4 I = sm.itf[j], C = sm.adj[j];
-                const c2 kj1 = kc2(medium_kz2<false>(p_hi, p_lo, sm.med[j + 1]));
+                const Kz2 kz1 = medium_kz2<false>(p_hi, p_lo, sm.med[j + 1]);
+                const c2 kj1 = kc2(kz1);
                 const float4 bv = ts.b[(bot ? NM : j) * kTeam + tid];
                 c2 G, b = czero(), kbar1 = czero(), rb = Bb, Xb_in = czero();
                 f2 accD = bc(0.f);
@@ -478,10 +481,10 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     kbar = cscla2(C.x, C.z, ga, kbar);
                     // k_j complete: accumulate conj(kbar) / k_j, or queue the
                     // interior-edge evaluation
-                    const f2 m2 = pfma(kj.re, kj.re, pmul(kj.im, kj.im));
-                    f2 inv = prcp(pmax(m2, bc(1e-30f)));
+                    f2 inv = yj;
                     if constexpr (edg) {
-                        const b2 edge{act[0] && m2.x < edge_u.x, act[1] && m2.y < edge_u.y};
+                        const f2 far = pmul(edge_u, yj); // |k_j|^2 < edge_u
+                        const b2 edge{act[0] && far.x > 1.f, act[1] && far.y > 1.f};
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const bool eh = h ? edge.y : edge.x;
@@ -516,11 +519,11 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 if constexpr (edg) Xb_up = Xb_in;
                 kbar = kbar1;
                 kj = kj1;
+                yj = kz1.y;
                 if constexpr (bot) { // backing medium n+1
                     const c2 kq = cmul2(kbar, kj);
-                    const f2 inv = prcp(pmax(pfma(kj.re, kj.re, pmul(kj.im, kj.im)), bc(1e-30f)));
-                    ur = pmul(kq.re, inv);
-                    ui = pneg(pmul(kq.im, inv));
+                    ur = pmul(kq.re, yj);
+                    ui = pneg(pmul(kq.im, yj));
                     add4(n + 1, bc(0.f), bc(0.f), ur, ui);
                     if constexpr (RES) res_sum = padd(res_sum, ur);
                 }
