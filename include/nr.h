@@ -186,9 +186,9 @@ nr_status nr_loglik_grad_res(nr_ctx *ctx, const nr_batch *batch, double *loglik,
  *   rho_out, iota_out: [n_stacks * nz] floats, stack-major (either may be
  *             NULL, not both).
  * Device batches run asynchronously on `stream`; host batches are staged
- * and synchronised.  The call uploads the stacks' parameter offsets into a
- * context buffer: calls of one context must not overlap on different
- * streams.  Non-finite parameters (or sigma < 0) raise
+ * and synchronised.  For stacks of different layer counts the call uploads
+ * their parameter offsets into a context buffer: calls of one context must
+ * not overlap on different streams.  Non-finite parameters (or sigma < 0) raise
  * NR_FLAG_NONFINITE_PARAM.  Errors: NR_EINVAL, NR_ECUDA. */
 nr_status nr_sld_profile(nr_ctx *ctx, const nr_batch *batch, const float *z, int32_t nz, float *rho_out,
                          float *iota_out, void *stream);

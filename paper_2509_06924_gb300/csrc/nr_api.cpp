@@ -1001,20 +1001,33 @@ nr_status nr_sld_profile(nr_ctx *ctx, const nr_batch *batch, const float *z, int
     if (!b->n_layers || !b->params) return fail(NR_EINVAL, "n_layers/params pointer is NULL");
     if (!z) return fail(NR_EINVAL, "z is NULL");
     if (!rho_out && !iota_out) return fail(NR_EINVAL, "rho_out and iota_out are both NULL");
-    std::vector<int64_t> off(S);
+    // Stacks of one layer count (the samples of one model) need no metadata on
+    // the device: the kernel takes the count itself.
+    const int n0 = b->n_layers[0];
+    bool same = true;
+    for (int s = 1; s < S; ++s) same &= b->n_layers[s] == n0;
+    std::vector<int64_t> off(same ? 0 : S);
     int64_t np = 0;
-    for (int s = 0; s < S; ++s) {
-        if (b->n_layers[s] < 0 || b->n_layers[s] > NR_MAX_LAYERS)
-            return fail(NR_EINVAL, "stack %d: n_layers %d outside [0, %d]", s, b->n_layers[s], NR_MAX_LAYERS);
-        off[s] = np;
-        np += 4 * (int64_t)b->n_layers[s] + 6;
+    if (same) {
+        if (n0 < 0 || n0 > NR_MAX_LAYERS)
+            return fail(NR_EINVAL, "stack %d: n_layers %d outside [0, %d]", 0, n0, NR_MAX_LAYERS);
+        np = (4 * (int64_t)n0 + 6) * S;
+    } else {
+        for (int s = 0; s < S; ++s) {
+            if (b->n_layers[s] < 0 || b->n_layers[s] > NR_MAX_LAYERS)
+                return fail(NR_EINVAL, "stack %d: n_layers %d outside [0, %d]", s, b->n_layers[s], NR_MAX_LAYERS);
+            off[s] = np;
+            np += 4 * (int64_t)b->n_layers[s] + 6;
+        }
     }
     NR_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    NR_CUDA(ctx->p_off.ensure(sizeof(int64_t) * S));
-    NR_CUDA(ctx->p_nl.ensure(sizeof(int32_t) * S));
-    NR_CUDA(cudaMemcpyAsync(ctx->p_off.p, off.data(), sizeof(int64_t) * S, cudaMemcpyHostToDevice, st));
-    NR_CUDA(cudaMemcpyAsync(ctx->p_nl.p, b->n_layers, sizeof(int32_t) * S, cudaMemcpyHostToDevice, st));
+    if (!same) {
+        NR_CUDA(ctx->p_off.ensure(sizeof(int64_t) * S));
+        NR_CUDA(ctx->p_nl.ensure(sizeof(int32_t) * S));
+        NR_CUDA(cudaMemcpyAsync(ctx->p_off.p, off.data(), sizeof(int64_t) * S, cudaMemcpyHostToDevice, st));
+        NR_CUDA(cudaMemcpyAsync(ctx->p_nl.p, b->n_layers, sizeof(int32_t) * S, cudaMemcpyHostToDevice, st));
+    }
     const size_t nout = sizeof(float) * (size_t)S * nz;
     const double *d_par = b->params;
     const float *d_z = z;
@@ -1029,8 +1042,9 @@ nr_status nr_sld_profile(nr_ctx *ctx, const nr_batch *batch, const float *z, int
         if (rho_out) { NR_CUDA(ctx->p_rho.ensure(nout)); d_rho = ctx->p_rho.as<float>(); }
         if (iota_out) { NR_CUDA(ctx->p_iota.ensure(nout)); d_iota = ctx->p_iota.as<float>(); }
     }
-    cudaError_t e = launch_profile(d_par, ctx->p_off.as<int64_t>(), ctx->p_nl.as<int32_t>(), S, d_z, nz, d_rho,
-                                   d_iota, ctx->d_status, ctx->sms, st);
+    cudaError_t e = launch_profile(d_par, same ? nullptr : ctx->p_off.as<int64_t>(),
+                                   same ? nullptr : ctx->p_nl.as<int32_t>(), n0, S, d_z, nz, d_rho, d_iota,
+                                   ctx->d_status, ctx->sms, st);
     if (e != cudaSuccess) return fail(NR_ECUDA, "profile launch: %s", cudaGetErrorString(e));
     if (b->memory == NR_MEM_HOST) {
         if (rho_out) NR_CUDA(cudaMemcpyAsync(rho_out, d_rho, nout, cudaMemcpyDeviceToHost, st));

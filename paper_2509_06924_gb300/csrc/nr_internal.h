@@ -145,8 +145,9 @@ cudaError_t launch_fp64(int mode, const KernelArgs &a, const QuadConst &qc, cuda
 cudaError_t launch_fp64_finalize(int mode, int n_stacks, const KernelArgs &a, cudaStream_t st);
 
 // ---- SLD profiles (nr_profile.cu) ----
-cudaError_t launch_profile(const double *params, const int64_t *par_off, const int32_t *n_layers, int n_stacks,
-                           const float *z, int nz, float *rho_out, float *iota_out, int32_t *status, int sms,
+// par_off, n_layers NULL: every stack has `n_same` layers
+cudaError_t launch_profile(const double *params, const int64_t *par_off, const int32_t *n_layers, int n_same,
+                           int n_stacks, const float *z, int nz, float *rho_out, float *iota_out, int32_t *status, int sms,
                            cudaStream_t st);
 
 // ---- co-fit samplers (nr_hmc.cu) ----

@@ -584,6 +584,38 @@ def test_sld_profile_parity(name, S):
     ctx.close()
 
 
+# Runs of 64 depths skip the error functions that are saturated over the whole
+# run: depths in any order (sorted, reversed, shuffled), fewer than one run
+# and one more than a whole number of them, more interfaces than a warp has
+# lanes, neighbouring roughnesses of very different width (a narrow interface
+# is passed while a wide one above it still counts), sharp steps and
+# zero-thickness layers.  Bound as for the workloads: FP32 rounding of the sum.
+@pytest.mark.parametrize("nz,order", [(1, "up"), (63, "down"), (65, "shuffled"), (640, "up"), (641, "shuffled")])
+def test_sld_profile_runs(nz, order):
+    rng = np.random.default_rng(nz)
+    stacks = []
+    for n in (0, 1, 5, 31, 32, 40, 64, 5, 12):
+        st = rand_stack(rng, n)
+        L = W.layout(n)
+        st[L["sigma"]] = rng.choice([0.0, 0.5, 3.0, 25.0, 80.0], n + 1)
+        if n >= 5:
+            st[L["d"]][2] = 0.0
+        stacks.append((n, st, 0))
+    q = W.log_grid(10, 0.01, 0.2)
+    wl = custom_workload(stacks, [(q, 0.05 * q.astype(np.float64))])
+    z = np.sort(rng.uniform(-300.0, 14000.0 if nz > 100 else 900.0, nz)).astype(np.float32)
+    z = z[::-1].copy() if order == "down" else rng.permutation(z) if order == "shuffled" else z
+    ctx = nr.Context(n_quad=wl.n_quad)
+    for sub in (wl, wl.subset([2, 7])):  # different layer counts, and one count
+        rho, iota = ctx.sld_profile(nr.Batch.from_workload(sub), torch.as_tensor(z, device="cuda"))
+        assert ctx.device_status() == 0
+        ref_r, ref_i = profile_ref(sub, z)
+        for s in range(sub.n_stacks):
+            assert np.max(np.abs(rho[s].cpu().numpy() - ref_r[s])) <= 2e-6 * max(np.max(np.abs(ref_r[s])), 1e-6)
+            assert np.max(np.abs(iota[s].cpu().numpy() - ref_i[s])) <= 2e-6 * max(np.max(np.abs(ref_i[s])), 1e-8)
+    ctx.close()
+
+
 def test_sld_profile_sharp_steps_host_batch_and_flags():
     d = [120.0, 35.0]
     rho = [0.0, 4.1e-6, -0.4e-6, 2.07e-6]
