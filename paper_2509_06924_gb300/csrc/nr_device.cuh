@@ -487,61 +487,71 @@ __device__ __forceinline__ float2 split_double(double v)
     return make_float2(hi, (float)(v - (double)hi));
 }
 
+// finite, by the exponent bits (no FP64 instruction)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// Thread j stages medium j / interface j / layer j; called by whole warps.
+// GB300 issues an FP64 instruction of a warp in 16 cycles of its SM, so the
+// staging (and the reductions below) use FP64 only where a result needs more
+// than one FP32 rounding of the parameter: with 48 such instructions a stack
+// here and 70 in the reductions, an item cost 0.8 us of its SM.
 template <int NM>
 __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, int32_t *status)
 {
-    // Thread j stages medium j / interface j / layer j.
-    if (tid <= n + 1) {
-        const int j = tid;
-        const double rho0 = p[n];
-        bool bad = false;
-        float4 lay = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (j >= 1) {
-            const double rj = p[n + j];
-            const double ij = p[2 * n + 2 + j - 1];
-            const float2 c = split_double(kFourPiD * (rj - rho0));
-            sm.med[j] = make_float4(c.x, c.y, (float)(kFourPiD * ij), (float)(kFourPiD * kFourPiD * ij * ij));
-            lay.w = (float)(kFourPiD * (ij + (j >= 2 ? p[2 * n + 2 + j - 2] : 0.0)));
-            bad |= !isfinite(rj) || !isfinite(ij);
-            if (j <= n) {
-                const double dj = p[j - 1];
-                const float2 d2 = split_double(dj * kTwoStepsD);
-                lay.x = d2.x;
-                lay.y = d2.y;
-                lay.z = (float)(-2.0 * kLog2ED * dj);
-                bad |= !isfinite(dj);
-            }
-        } else {
-            bad |= !isfinite(rho0);
-        }
-        if (j <= n) {
-            const double iot_j = j >= 1 ? p[2 * n + 2 + j - 1] : 0.0;
-            const double iot_j1 = p[2 * n + 2 + j];
-            const double sig = p[3 * n + 3 + j];
-            const float Nr = (float)(kFourPiD * (p[n + j + 1] - p[n + j]));
-            const float Ni = (float)(kFourPiD * (iot_j - iot_j1));
-            const float s = (float)(-2.0 * sig * sig);
-            sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig * sig));
-            sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, j < n ? (float)(2.0 * p[j]) : 0.f);
-            sm.sig[j] = (float)sig;
-            bad |= !isfinite(sig);
-            // |s Im(k_j k_{j+1})| <= -s (D / 2 + sqrt(5 m a) + a) with
-            // D = |Re N|, a the larger 4 pi iota of the two media, m = max(D, a):
-            // with k^2 = u + i a of each, 2 Im^2 = |z z'| - Re(z z') is at most
-            // D^2 / 2 where u and u' differ in sign, plus |u| a' + |u'| a
-            // + 2 a a'; for |u| > 4 m of one sign it is below (0.6 (a + a'))^2 x 2
-            const float D = fabsf(Nr), a = (float)kFourPiD * fmaxf(fabsf((float)iot_j), fabsf((float)iot_j1));
-            const float bound = -s * (0.5f * D + sqrtf(5.f * fmaxf(D, a) * a) + 1.2f * a);
-            if (!(bound <= kNcSmall)) sm.nc_big = 1; // every writer stores the same value
-        }
-        sm.lay[j] = lay;
-        if (j == 0) {
-            sm.scale = (float)p[4 * n + 4];
-            sm.bkg = (float)p[4 * n + 5];
-            bad |= !isfinite(p[4 * n + 4]) || !isfinite(p[4 * n + 5]);
-        }
-        if (bad) atomicOr(status, NR_FLAG_NONFINITE_PARAM);
+    const int j = tid, lane = tid & 31;
+    if (tid - lane > n + 1) return;
+    const bool on = j <= n + 1, med = on && j >= 1, itf = j <= n, layer = med && itf;
+    const double rho0 = p[n], rj = on ? p[n + j] : 0.0, ij = med ? p[2 * n + 1 + j] : 0.0;
+    const double dj = layer ? p[j - 1] : 0.0, sig = itf ? p[3 * n + 3 + j] : 0.0;
+    const float aj = (float)(kFourPiD * ij); // 4 pi iota_j; its neighbours'
+    float aup = __shfl_up_sync(kFull, aj, 1), adn = __shfl_down_sync(kFull, aj, 1);
+    if (lane == 0 && j >= 2 && on) aup = (float)(kFourPiD * p[2 * n + j]);
+    if (lane == 31 && itf) adn = (float)(kFourPiD * p[2 * n + 2 + j]);
+    bool bad = !finite_bits(rj) || !finite_bits(ij) || !finite_bits(dj) || !finite_bits(sig);
+    if (med) {
+        const float2 c = split_double(kFourPiD * (rj - rho0));
+        sm.med[j] = make_float4(c.x, c.y, aj, aj * aj);
     }
+    if (on) {
+        const float2 d2 = split_double(dj * kTwoStepsD);
+        sm.lay[j] = make_float4(d2.x, d2.y, (float)(-2.0 * kLog2ED * dj), j >= 1 ? aup + aj : 0.f);
+    }
+    if (itf) {
+        const float dn = j < n ? 2.f * (float)p[j] : 0.f;
+        const float Nr = (float)(kFourPiD * (p[n + j + 1] - rj)), Ni = aj - adn;
+        const double sig2 = sig * sig;
+        const float s = -2.f * (float)sig2;
+        sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig2));
+        sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, dn);
+        sm.sig[j] = (float)sig;
+        // |s Im(k_j k_{j+1})| <= -s (D / 2 + sqrt(5 m a) + a) with
+        // D = |Re N|, a the larger 4 pi iota of the two media, m = max(D, a):
+        // with k^2 = u + i a of each, 2 Im^2 = |z z'| - Re(z z') is at most
+        // D^2 / 2 where u and u' differ in sign, plus |u| a' + |u'| a
+        // + 2 a a'; for |u| > 4 m of one sign it is below (0.6 (a + a'))^2 x 2
+        const float D = fabsf(Nr), a = fmaxf(fabsf(aj), fabsf(adn));
+        const float bound = -s * (0.5f * D + sqrtf(5.f * fmaxf(D, a) * a) + 1.2f * a);
+        if (!(bound <= kNcSmall)) sm.nc_big = 1; // every writer stores the same value
+    }
+    if (j == 0) {
+        const double scale = p[4 * n + 4], bkg = p[4 * n + 5];
+        sm.scale = (float)scale;
+        sm.bkg = (float)bkg;
+        bad |= !finite_bits(scale) || !finite_bits(bkg);
+    }
+    if (bad) atomicOr(status, NR_FLAG_NONFINITE_PARAM);
+}
+
+// v0 + v1 + v2 + v3 (+ lo) to FP64 accuracy of the floats' sum: error-free
+// transformations in FP32 and one FP64 addition
+__device__ __forceinline__ double sum4(float v0, float v1, float v2, float v3, float lo)
+{
+    float s1, e1, s2, e2, s, e;
+    two_sum(v0, v1, s1, e1);
+    two_sum(v2, v3, s2, e2);
+    two_sum(s1, s2, s, e);
+    const float err = __fadd_rn(e, __fadd_rn(e1, e2));
+    return (double)s + (double)__fadd_rn(err == err ? err : 0.f, lo); // an infinite sum stays infinite
 }
 
 // Convert a stack's raw sums into outputs (loglik, packed gradient).
@@ -556,24 +566,19 @@ __device__ void finalize_stack(const double *raw, int n, const double *p, int s,
     const double twoPi = 6.283185307179586476925286766559;
     double *g = grad_out + par_off;
     for (int i = tid; i < 4 * n + 6; i += nthreads) {
+        // d_j: 2 raw; rho_j, iota_j (j >= 1): -2 pi raw; sigma_j: -4 sigma_j raw;
+        // scale, bkg: raw.  One multiplication for all of them.
+        double coef = i < n ? 2.0 : i < 3 * n + 3 ? -twoPi : 1.0;
         double v;
-        if (i < n) {
-            v = 2.0 * raw[i];                                  // d_j
-        } else if (i == n) {                                   // rho_0 = -sum rho_j
-            double acc = 0.0;
-            for (int j = 1; j <= n + 1; ++j) acc += raw[n + j - 1];
-            v = twoPi * acc;
-        } else if (i < 2 * n + 2) {
-            v = -twoPi * raw[n + (i - n) - 1];                 // rho_j, j >= 1
-        } else if (i < 3 * n + 3) {
-            v = -twoPi * raw[2 * n + 1 + (i - (2 * n + 2))];   // iota_j
-        } else if (i < 4 * n + 4) {
-            const int j = i - (3 * n + 3);
-            v = -4.0 * p[3 * n + 3 + j] * raw[3 * n + 2 + j];  // sigma_j
+        if (i >= 3 * n + 3 && i < 4 * n + 4) coef = -4.0 * p[i];
+        if (i == n) {                                          // rho_0 = -sum rho_j
+            v = 0.0;
+            for (int j = 1; j <= n + 1; ++j) v += raw[n + j - 1];
+            v = -v;
         } else {
-            v = raw[i];                                        // scale, bkg
+            v = raw[i < n || i >= 4 * n + 4 ? i : i - 1];
         }
-        g[i] = v;
+        g[i] = coef * v;
     }
 }
 

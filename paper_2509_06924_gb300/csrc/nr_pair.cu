@@ -115,8 +115,9 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
     __shared__ __align__(16) float sh_wR[2][WRN];
     __shared__ float4 sh_qd[CAPQ];                      // (Q/2, dQ/2, R_obs, 1/err) per staged Q point
     __shared__ float2 sh_rs[LIK ? CAPQ : 1];            // (residual, S) per staged Q point
-    __shared__ double sh_red[WARPS][32];
-    __shared__ double sh_redd[WARPS][4];
+    static_assert(WARPS == 4, "sum4 adds the warps' sums");
+    __shared__ float sh_red[WARPS][32];
+    __shared__ float sh_redd[WARPS][5]; // loglik (hi), d/dscale, d/dbkg, d/d ln f; loglik (lo)
     __shared__ double sh_raw[NRAW];
     __shared__ int sh_item;
     __shared__ int sh_last;
@@ -163,18 +164,19 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
     for (int i = tid; i < 2 * WRN; i += BLOCK) (&sh_wR[0][0])[i] = 0.f; // padding stays 0
     for (int i = tid; i < 2 * kTabN; i += BLOCK) sh_cs[i] = qc.cs_tab[i];  // read after the item barrier
 
-    for (;;) {
-        if (tid == 0) {
-            sh_item = atomicAdd(&ka.ticket[0], 1);
-            sm.nc_big = 0;
-        }
-        __syncthreads();
-        const int item = sh_item;
-        if (item >= ka.n_items) break;
+    // the first item of a CTA is its own, the others come by ticket
+    for (int item = blockIdx.x; item < ka.n_items;) {
         const WorkItem wi = ka.items[item];
+        if (tid == 0) sm.nc_big = 0;
+        __syncthreads();
         if constexpr (NR_DEBUG) {
             if (!item_in_bounds(ka, wi, NMAX)) { // uniform over the block
-                if (tid == 0) atomicOr(ka.status, NR_FLAG_DEBUG_BOUNDS);
+                if (tid == 0) {
+                    atomicOr(ka.status, NR_FLAG_DEBUG_BOUNDS);
+                    sh_item = gridDim.x + atomicAdd(&ka.ticket[0], 1);
+                }
+                __syncthreads();
+                item = sh_item;
                 __syncthreads(); // every thread has read sh_item
                 continue;
             }
@@ -560,6 +562,8 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             } // LIK
         }
 
+        if (tid == 0) sh_item = gridDim.x + atomicAdd(&ka.ticket[0], 1); // its latency overlaps the reductions
+
         if constexpr (LIK) {
             if constexpr (GRAD) {
                 if (eq_cnt > 0) {
@@ -577,7 +581,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     float v = accr[t].x + accr[t].y;
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-                    if (lane == 0) sh_red[warp][t] = (double)v;
+                    if (lane == 0) sh_red[warp][t] = v;
                 }
                 __syncthreads();
                 if (tid < NACC) {
@@ -587,13 +591,8 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                                   : t < 2 * NM + 1 ? (t - NM <= n ? n + (t - NM) : -1)
                                   : t < 3 * NM + 2 ? (t - 2 * NM - 1 <= n ? 2 * n + 1 + (t - 2 * NM - 1) : -1)
                                                    : (t - 3 * NM - 2 <= n ? 3 * n + 2 + (t - 3 * NM - 2) : -1);
-                    if (i >= 0) {
-                        double s = 0.0;
-                        for (int w = 0; w < WARPS; ++w) s += sh_red[w][t];
-                        sh_raw[i] = s;
-                    }
+                    if (i >= 0) sh_raw[i] = sum4(sh_red[0][t], sh_red[1][t], sh_red[2][t], sh_red[3][t], 0.f);
                 }
-                __syncthreads();
             }
             {   // loglik (float pair), d/dscale, d/dbkg, d/d ln(dQ scale)
                 float h = ll_hi, l = ll_lo, a1 = gsc_acc, a2 = gbk_acc, a3 = gres_acc.x + gres_acc.y;
@@ -609,17 +608,17 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     if constexpr (RES) a3 += __shfl_xor_sync(kFull, a3, o);
                 }
                 if (lane == 0) {
-                    sh_redd[warp][0] = (double)h + (double)l;
+                    sh_redd[warp][0] = h;
                     sh_redd[warp][1] = a1;
                     sh_redd[warp][2] = a2;
                     sh_redd[warp][3] = a3;
+                    sh_redd[warp][4] = l;
                 }
             }
             __syncthreads();
             if (tid < (RES ? 4 : 3)) {
-                double s = 0.0;
-                for (int w = 0; w < WARPS; ++w) s += sh_redd[w][tid];
-                sh_raw[4 * n + 3 + tid] = s;
+                const float lo = tid == 0 ? (sh_redd[0][4] + sh_redd[1][4]) + (sh_redd[2][4] + sh_redd[3][4]) : 0.f;
+                sh_raw[4 * n + 3 + tid] = sum4(sh_redd[0][tid], sh_redd[1][tid], sh_redd[2][tid], sh_redd[3][tid], lo);
             }
             __syncthreads();
             const int nout = GRAD ? 4 * n + (RES ? 7 : 6) : 1;
@@ -630,9 +629,9 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             } else {
                 double *slot = ka.partials + si.part_base + (int64_t)wi.chunk * n_slot(n);
                 for (int i = tid; i < nout; i += BLOCK) slot[off0 + i] = sh_raw[off0 + i];
-                __threadfence();
                 __syncthreads();
                 if (tid == 0) {
+                    __threadfence(); // after the barrier: covers the whole CTA's slot
                     const int prev = atomicAdd(&ka.stack_done[wi.stack], 1);
                     sh_last = prev == si.n_chunks - 1;
                 }
@@ -641,6 +640,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     __threadfence();
                     for (int i = tid; i < nout; i += BLOCK) {
                         double s = 0.0;
+#pragma unroll 8
                         for (int c = 0; c < si.n_chunks; ++c)
                             s += __ldcg(ka.partials + si.part_base + (int64_t)c * n_slot(n) + off0 + i);
                         sh_raw[off0 + i] = s;
@@ -652,6 +652,8 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                 }
             }
         } // LIK
+        __syncthreads();
+        item = sh_item;
         __syncthreads(); // sm / sh_raw / sh_item / sh_wR reused by the next item
     }
     // last CTA out resets the queue for the next launch

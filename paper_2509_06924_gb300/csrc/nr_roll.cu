@@ -68,7 +68,7 @@ struct TeamSmem {
     float2 eq[kTeamWarps][3][kEqCap];            // edge queue: node k_0 (hi, lo), Z, Xbar_{j-1}
     float eqr[RES ? kTeamWarps : 1][RES ? kEqCap : 1]; // k_0 dk_0 / d ln f of an entry
     int eqj[kTeamWarps][kEqCap];                 // its medium
-    double redd[kTeamWarps][4];
+    float redd[kTeamWarps][5];                   // loglik (hi), d/dscale, d/dbkg, d/d ln f; loglik (lo)
     double raw[4 * NM + 7];
     StackSmem<NM> sm;
     int item, last;
@@ -218,14 +218,15 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
     int item = team * gridDim.x + blockIdx.x;
     for (; item < ka.n_items;) {
         const WorkItem wi = ka.items[item];
-        if (tid == 0) {
-            ts.item = workers + atomicAdd(&ka.ticket[0], 1);
-            sm.nc_big = 0;
-        }
+        if (tid == 0) sm.nc_big = 0;
         team_sync(team);
         if constexpr (NR_DEBUG) {
             if (!item_in_bounds(ka, wi, NMAX)) { // uniform over the team
-                if (tid == 0) atomicOr(ka.status, NR_FLAG_DEBUG_BOUNDS);
+                if (tid == 0) {
+                    atomicOr(ka.status, NR_FLAG_DEBUG_BOUNDS);
+                    ts.item = workers + atomicAdd(&ka.ticket[0], 1);
+                }
+                team_sync(team);
                 item = ts.item;
                 team_sync(team); // every thread has read ts.item
                 continue;
@@ -540,6 +541,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             else sweep(std::false_type{});
             if constexpr (RES) gres_acc = pfma(wres, pfma(k0h, res_sum, res_k0), gres_acc);
         }
+        if (tid == 0) ts.item = workers + atomicAdd(&ka.ticket[0], 1); // its latency overlaps the reductions
         if (eq_cnt > 0) eq_drain();
 
         // ---- team reduction of the item's partial sums into raw ----
@@ -550,13 +552,13 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             // step of the sum, and which lane of the quads holds it
             const int step = i < n ? i : i < 2 * n + 1 ? i - n + 1 : i < 3 * n + 2 ? i - 2 * n : i - 3 * n - 2;
             const int of = i < n ? 0 : i < 2 * n + 1 ? 1 : i < 3 * n + 2 ? 3 : 2;
-            double sum = 0.0;
+            float w4[kTeamWarps];
 #pragma unroll
             for (int w = 0; w < kTeamWarps; ++w) {
                 const float *v = ts.acc[w] + step * 32 + of;
-                sum += (double)(((v[0] + v[4]) + (v[8] + v[12])) + ((v[16] + v[20]) + (v[24] + v[28])));
+                w4[w] = ((v[0] + v[4]) + (v[8] + v[12])) + ((v[16] + v[20]) + (v[24] + v[28]));
             }
-            ts.raw[i] = sum;
+            ts.raw[i] = sum4(w4[0], w4[1], w4[2], w4[3], 0.f);
         }
         {   // loglik (float pair), d/dscale, d/dbkg, d/d ln(dQ scale)
             float h = ll_hi, l = ll_lo, a1 = gsc_acc, a2 = gbk_acc, a3 = gres_acc.x + gres_acc.y;
@@ -572,17 +574,17 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 if constexpr (RES) a3 += __shfl_xor_sync(kFull, a3, o);
             }
             if (lane == 0) {
-                ts.redd[warp][0] = (double)h + (double)l;
+                ts.redd[warp][0] = h;
                 ts.redd[warp][1] = a1;
                 ts.redd[warp][2] = a2;
                 ts.redd[warp][3] = a3;
+                ts.redd[warp][4] = l;
             }
         }
         team_sync(team);
         if (tid < (RES ? 4 : 3)) {
-            double s = 0.0;
-            for (int w = 0; w < kTeamWarps; ++w) s += ts.redd[w][tid];
-            ts.raw[4 * n + 3 + tid] = s;
+            const float lo = tid == 0 ? (ts.redd[0][4] + ts.redd[1][4]) + (ts.redd[2][4] + ts.redd[3][4]) : 0.f;
+            ts.raw[4 * n + 3 + tid] = sum4(ts.redd[0][tid], ts.redd[1][tid], ts.redd[2][tid], ts.redd[3][tid], lo);
         }
         item = ts.item; // the next item, before its slot is written again
         team_sync(team);
@@ -592,9 +594,9 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         } else {
             double *slot = ka.partials + si.part_base + (int64_t)wi.chunk * n_slot(n);
             for (int i = tid; i < nout; i += kTeam) slot[i] = ts.raw[i];
-            __threadfence();
             team_sync(team);
             if (tid == 0) {
+                __threadfence(); // after the barrier: covers the whole team's slot
                 const int prev = atomicAdd(&ka.stack_done[wi.stack], 1);
                 ts.last = prev == si.n_chunks - 1;
             }
@@ -603,6 +605,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 __threadfence();
                 for (int i = tid; i < nout; i += kTeam) {
                     double s = 0.0;
+#pragma unroll 8
                     for (int c = 0; c < si.n_chunks; ++c)
                         s += __ldcg(ka.partials + si.part_base + (int64_t)c * n_slot(n) + i);
                     ts.raw[i] = s;
