@@ -307,18 +307,27 @@ bool same_meta(const Plan &p, const nr_batch *b, int K)
 
 // Cutting stacks into Q-range chunks.  The register buckets of a work list
 // run concurrently, so their chunk lengths are chosen together: for a bound
-// B on the cost of any one item, every bucket takes its longest chunk (a
+// B on the time of any one item, every bucket takes its longest chunk (a
 // multiple of its tile, or the whole dataset) whose items stay within B, and
-// the estimated makespan is Graham's bound for longest-first queues, the
-// summed cost of all items / resident CTAs + B.  An item costs (n + 1) x its
-// Q points x K layer-evaluations plus a fixed overhead (queue ticket,
-// staging, reductions, output) of about kItemOverhead layer-evaluations
-// (measured: about 4 us of a CTA's time on the one-layer kernels), twice
-// that for a chunk of a cut stack (partial sums, arrival counter, the last
-// arriver's sum).  The best B must beat whole stacks by 10 %; batches with
-// kChunkWaves stacks per resident CTA keep whole stacks without the search.
+// the launch's time is estimated from a model of one SM, in microseconds on
+// GB300, fitted to launches of 1 to 4096 stacks of one and ten layers:
+//   - a tile (256 evaluations) of a stack with n layers takes (n + 1) x
+//     0.26 us of an SM that is full (0.18 up to two layers, 0.11 without a
+//     gradient);
+//   - an item costs 1.5 us of it besides (0.85 and 0.3): staging,
+//     reductions, output;
+//   - k items at once on an SM reach a share kShare[k] of its full rate;
+//   - cutting stacks at all adds the partial sums' round trip through memory.
+// So few stacks are cut until every SM has a few items, and no further: the
+// rule before, a fixed overhead per item and no loss at low concurrency,
+// took 29 us for the gradient of 300 one-layer stacks (whole 24 us) and 30
+// for their log-likelihood (whole 18), 137 us for 100 chains of three
+// ten-layer contrasts (now 120).  Whole stacks are kept unless another choice
+// is 3 % faster; batches with kChunkWaves stacks per resident CTA keep them
+// without the search.
 constexpr int64_t kChunkWaves = 8;
-constexpr double kItemOverhead = 1000.0;
+constexpr double kShare[] = {0.55, 0.55, 0.77, 0.91, 0.97, 1.0};
+constexpr double kCutCost = 4.0;
 
 struct GroupSpan {
     int nmax;
@@ -327,30 +336,43 @@ struct GroupSpan {
     int64_t resident;
 };
 
-// One chunk length of a group with its summed item cost, largest item cost
-// and item count
+// Times of a bucket's items in us: a tile per (n + 1), an item besides
+struct ItemCost {
+    double tile, item;
+};
+ItemCost item_cost(int mode, int nmax)
+{
+    if (!is_grad_mode(mode)) return {0.11, 0.3};
+    return nmax <= 2 ? ItemCost{0.18, 0.85} : ItemCost{0.26, 1.5};
+}
+
+// One chunk length of a group: its items' summed time, largest item (us) and count
 struct ChunkCand {
     int64_t chunk;
     double total, big;
+    int64_t items;
 };
 
-std::vector<int64_t> choose_chunks(const Plan &pl, const std::vector<int> &order, const std::vector<GroupSpan> &gs)
+std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std::vector<int> &order,
+                                   const std::vector<GroupSpan> &gs)
 {
     std::vector<int64_t> whole(gs.size(), 1);
     int64_t nst = 0;
     double res_w = 0.0, w_sum = 0.0;
     std::vector<std::vector<ChunkCand>> cands(gs.size());
-    const double O = kItemOverhead / std::max(pl.K, 1); // in (n + 1) x Q units
     auto dlen = [&](int s) { return pl.q_off[pl.dataset[s] + 1] - pl.q_off[pl.dataset[s]]; };
     auto cost_of = [&](const GroupSpan &g, int64_t chunk) {
-        ChunkCand c{chunk, 0.0, 0.0};
+        const ItemCost ic = item_cost(mode, g.nmax);
+        ChunkCand c{chunk, 0.0, 0.0, 0};
         for (size_t i = g.i0; i < g.i1; ++i) {
             const int s = order[i];
-            const int64_t len = dlen(s);
-            const int64_t nch = std::max<int64_t>(1, (len + chunk - 1) / chunk);
-            const double o = nch > 1 ? 2.0 * O : O, w = pl.n_layers[s] + 1.0;
-            c.total += w * (double)len + (double)nch * o;
-            c.big = std::max(c.big, w * (double)std::min(chunk, std::max<int64_t>(len, 1)) + o);
+            const int64_t len = std::max<int64_t>(dlen(s), 1), ch = std::min(chunk, len);
+            const int64_t nch = (len + ch - 1) / ch, rest = len - (nch - 1) * ch;
+            const double w = ic.tile * (pl.n_layers[s] + 1.0);
+            const int64_t t = (ch + g.tile_q - 1) / g.tile_q, tr = (rest + g.tile_q - 1) / g.tile_q;
+            c.total += w * (double)((nch - 1) * t + tr) + (double)nch * ic.item;
+            c.big = std::max(c.big, w * (double)t + ic.item);
+            c.items += nch;
         }
         return c;
     };
@@ -372,9 +394,28 @@ std::vector<int64_t> choose_chunks(const Plan &pl, const std::vector<int> &order
         // dozen candidates however long the datasets are)
         for (int64_t mt = 1; mt * gs[k].tile_q < whole[k]; mt = mt < 16 ? mt + 1 : mt + (mt + 3) / 4)
             cands[k].push_back(cost_of(gs[k], mt * gs[k].tile_q));
-    // the makespan estimate for a bound B on the largest item
+    // items of mean time `mean` and largest `big`, `n` of them: full rounds of
+    // R at the full rate, then the last round at its own concurrency
+    auto time_of = [&](double total, double big, double n) {
+        const double mean = total / std::max(n, 1.0);
+        const double rounds = std::floor(n / R), rem = n - rounds * R;
+        double t = rounds * R * mean / sms;
+        if (rem > 0.0) {
+            const int k = (int)std::ceil(rem / sms);
+            t += (rounds > 0.0 ? mean : std::max(mean, big)) * k / kShare[std::min(k, 5)];
+        }
+        return std::max(t, big / kShare[1]);
+    };
+    // several buckets' launches share the SMs a CTA at a time: each one's last
+    // items hold theirs while the others wait
+    auto time_all = [&](double total, double big, double n, double bigs) {
+        const double t = time_of(total, big, n);
+        return gs.size() > 1 ? std::max(t, total / sms + 0.6 * bigs) : t;
+    };
+    // the estimate for a bound B on the largest item
     auto est = [&](double B, std::vector<int64_t> *pick) {
-        double total = 0.0, big = 0.0;
+        double total = 0.0, big = 0.0, n = 0.0, bigs = 0.0;
+        bool cut = false;
         for (size_t k = 0; k < gs.size(); ++k) {
             const ChunkCand *sel = nullptr;
             for (const ChunkCand &c : cands[k])
@@ -382,18 +423,23 @@ std::vector<int64_t> choose_chunks(const Plan &pl, const std::vector<int> &order
             if (!sel) return -1.0;
             total += sel->total;
             big = std::max(big, sel->big);
+            bigs += sel->big;
+            n += (double)sel->items;
+            cut |= sel->chunk < whole[k];
             if (pick) (*pick)[k] = sel->chunk;
         }
-        return total / R + big;
+        return time_all(total, big, n, bigs) + (cut ? kCutCost : 0.0);
     };
     double whole_est = 0.0;
     {
-        double total = 0.0, big = 0.0;
+        double total = 0.0, big = 0.0, n = 0.0, bigs = 0.0;
         for (size_t k = 0; k < gs.size(); ++k) {
             total += cands[k][0].total;
             big = std::max(big, cands[k][0].big);
+            bigs += cands[k][0].big;
+            n += (double)cands[k][0].items;
         }
-        whole_est = total / R + big;
+        whole_est = time_all(total, big, n, bigs);
     }
     double best_est = whole_est, best_B = -1.0;
     for (size_t k = 0; k < gs.size(); ++k)
@@ -404,7 +450,7 @@ std::vector<int64_t> choose_chunks(const Plan &pl, const std::vector<int> &order
                 best_B = c.big;
             }
         }
-    if (best_B < 0.0 || best_est >= 0.9 * whole_est) return whole;
+    if (best_B < 0.0 || best_est >= 0.97 * whole_est) return whole;
     std::vector<int64_t> pick(gs.size(), 1);
     est(best_B, &pick);
     return pick;
@@ -475,7 +521,7 @@ nr_status build_worklist(nr_ctx *ctx, Plan &pl, int mode, WorkList &wl)
         i0 = i1;
     }
     std::vector<int64_t> chunks = ctx->opt.chunk_q > 0 ? std::vector<int64_t>(spans.size(), ctx->opt.chunk_q)
-                                                       : choose_chunks(pl, order, spans);
+                                                       : choose_chunks(pl, mode, ctx->sms, order, spans);
     int64_t part = 0;
     wl.chunk_q = 0;
     for (size_t k = 0; k < spans.size(); ++k) {

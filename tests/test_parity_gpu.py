@@ -412,6 +412,28 @@ def test_chunk_choice_follows_the_makespan_estimate():
     assert_parity(wl, run_gpu(wl), run_oracle(wl))
 
 
+@pytest.mark.parametrize("n,S,whole", [(1, 300, True), (1, 1, False), (10, 100, False), (10, 608, True)])
+def test_chunk_choice_of_small_batches(n, S, whole):
+    """A few hundred short stacks stay whole (one or two per SM are fast
+    enough), a single one or long stacks that leave SMs idle are cut, long
+    ones that fill the SMs are not; the first stacks keep parity."""
+    rng = np.random.default_rng(n * 1000 + S)
+    q = W.log_grid(225 if n > 1 else 200, 0.005, 0.3)
+    wl = custom_workload([(n, rand_stack(rng, n), 0) for _ in range(S)], [(q, 0.05 * q.astype(np.float64))])
+    ctx = nr.Context(n_quad=wl.n_quad)
+    b = nr.Batch.from_workload(wl)
+    items = sum(g["items"] for g in ctx.plan_groups(b, grad=True))
+    assert (items == S) == whole
+    ll, g = (t.cpu().numpy() for t in ctx.loglik_grad(b))
+    assert ctx.device_status() == 0
+    ctx.close()
+    k = min(S, 4)
+    sub = wl.subset(np.arange(k))
+    ref = run_oracle(sub, modes=("grad",))
+    errs = stack_errors(sub, {"ll_g": ll[:k], "g": g[:sub.params.size]}, ref)
+    check_bounds(sub, errs, {"loglik_g": TOL_LL, "grad": TOL_G})
+
+
 def test_host_memory_calls_match_device_calls():
     wl = W.make_workload("uneven", n_stacks=20)
     ctx = nr.Context(n_quad=wl.n_quad)
