@@ -264,7 +264,7 @@ struct nr_sampler {
     std::vector<int64_t> q_off;
     nr_batch batch{};
     DevBuf d_src, d_val, d_lo, d_hi, d_tie_ptr, d_tie_slot, d_params, d_ll, d_gpk, d_mom, d_u0, d_H0, d_lp0;
-    DevBuf d_vu, d_vg, d_vlp, d_vpart; // variational step: u = mu + L e, d log pi / du, log pi, ELBO part
+    DevBuf d_vu, d_vg, d_vpart;        // variational step: u = mu + L e, d log pi / du, ELBO part
     DevBuf d_vbias;                    // Adam bias corrections of the current iteration (2 doubles)
     int res_param = -1;                // free parameter scaling every dQ (-1: none)
     DevBuf d_dqs, d_gres;              // per stack: that scale, d loglik / d ln(scale)
@@ -1173,7 +1173,6 @@ nr_status nr_sampler_create(nr_ctx *ctx, const nr_cofit_model *m, nr_sampler **o
     NR_CUDA(S.d_lp0.ensure(sizeof(double) * C));
     NR_CUDA(S.d_vu.ensure(sizeof(double) * (size_t)C * P));
     NR_CUDA(S.d_vg.ensure(sizeof(double) * (size_t)C * P));
-    NR_CUDA(S.d_vlp.ensure(sizeof(double) * C));
     NR_CUDA(S.d_vpart.ensure(sizeof(double) * C));
     NR_CUDA(S.d_vbias.ensure(sizeof(double) * 2));
     S.res_param = m->res_param;
@@ -1243,17 +1242,23 @@ CofitStageArgs stage_args(nr_sampler *S, double *u, int stage)
     return a;
 }
 
-// log-likelihood and packed gradient of every stack at the chains' u
+// log-likelihood and packed gradient of the sampler's stacks as gathered
+nr_status sampler_likelihood(nr_sampler *S, cudaStream_t st)
+{
+    if (S->res_param >= 0)
+        return compute(S->ctx, &S->batch, kGradRes, nullptr, S->d_ll.as<double>(), S->d_gpk.as<double>(),
+                       S->d_gres.as<double>(), st, S->d_dqs.as<double>());
+    return compute(S->ctx, &S->batch, kGrad, nullptr, S->d_ll.as<double>(), S->d_gpk.as<double>(), nullptr, st);
+}
+
+// the same at the chains' u
 nr_status sampler_eval(nr_sampler *S, const double *u, cudaStream_t st)
 {
     cudaError_t e = launch_cofit_gather(u, S->C, S->P, S->NS, S->d_src.as<int32_t>(), S->d_val.as<double>(),
                                         S->d_lo.as<double>(), S->d_hi.as<double>(), S->d_params.as<double>(),
                                         S->res_param, S->NC, S->d_dqs.as<double>(), st);
     if (e != cudaSuccess) return fail(NR_ECUDA, "sampler gather: %s", cudaGetErrorString(e));
-    if (S->res_param >= 0)
-        return compute(S->ctx, &S->batch, kGradRes, nullptr, S->d_ll.as<double>(), S->d_gpk.as<double>(),
-                       S->d_gres.as<double>(), st, S->d_dqs.as<double>());
-    return compute(S->ctx, &S->batch, kGrad, nullptr, S->d_ll.as<double>(), S->d_gpk.as<double>(), nullptr, st);
+    return sampler_likelihood(S, st);
 }
 } // namespace
 
@@ -1307,20 +1312,24 @@ nr_status nr_vi_step(nr_sampler *S, double *phi, double *adam_m, double *adam_v,
     NR_CUDA(cudaSetDevice(S->ctx->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     double *u = S->d_vu.as<double>();
+    CofitGatherArgs ga{};
+    ga.NS = S->NS;
+    ga.NC = S->NC;
+    ga.res_param = S->res_param;
+    ga.src = S->d_src.as<int32_t>();
+    ga.val = S->d_val.as<double>();
+    ga.lo = S->d_lo.as<double>();
+    ga.hi = S->d_hi.as<double>();
+    ga.params = S->d_params.as<double>();
+    ga.dq_scale = S->d_dqs.as<double>();
     cudaError_t e = launch_vi_sample(phi, eps, S->C, S->P, u, S->d_vpart.as<double>(), t, opt->beta1, opt->beta2,
-                                     S->d_vbias.as<double>(), st);
+                                     S->d_vbias.as<double>(), ga, st);
     if (e != cudaSuccess) return fail(NR_ECUDA, "vi sample: %s", cudaGetErrorString(e));
-    nr_status r = sampler_eval(S, u, st);
+    nr_status r = sampler_likelihood(S, st);
     if (r != NR_OK) return r;
-    CofitStageArgs a = stage_args(S, u, kStageLogp);
-    a.logp_out = S->d_vlp.as<double>();
-    a.grad_out = S->d_vg.as<double>();
-    e = launch_cofit_stage(a, st);
-    if (e == cudaSuccess)
-        e = launch_vi_adam(phi, adam_m, adam_v, eps, S->d_vg.as<double>(), S->d_vlp.as<double>(),
-                           S->d_vpart.as<double>(), S->C, S->P, S->d_vbias.as<double>(), opt->lr, opt->beta1,
-                           opt->beta2, opt->eps, elbo,
-                           st);
+    e = launch_vi_adam(phi, adam_m, adam_v, eps, S->d_vg.as<double>(), S->d_vpart.as<double>(),
+                       S->d_vbias.as<double>(), opt->lr, opt->beta1, opt->beta2, opt->eps, elbo,
+                       stage_args(S, u, kStageLogp), st);
     if (e != cudaSuccess) return fail(NR_ECUDA, "vi step: %s", cudaGetErrorString(e));
     return NR_OK;
 }

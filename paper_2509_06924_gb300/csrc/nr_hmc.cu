@@ -28,6 +28,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "nr_cofit.cuh"
 #include "nr_internal.h"
 
 namespace nrimpl {
@@ -74,25 +75,12 @@ __global__ void cofit_stage_kernel(CofitStageArgs a)
     if (c >= a.C) return;
     const int P = a.P;
     double *u = a.u + (int64_t)c * P;
-    const double *gpk = a.gpk + (int64_t)c * a.NS;
     // log pi: the contrasts' log-likelihoods plus the prior/Jacobian terms
     double lp = 0.0, kin0 = 0.0, kin1 = 0.0;
     for (int i = lane; i < a.n_contrast; i += 32) lp += a.ll[(int64_t)c * a.n_contrast + i];
     for (int k = lane; k < P; k += 32) {
         const double uk = u[k];
-        const double s = 1.0 / (1.0 + exp(-uk));
-        const double au = fabs(uk);
-        lp += -au - 2.0 * log1p(exp(-au));
-        double gt = 0.0;
-        for (int t = a.tie_ptr[k]; t < a.tie_ptr[k + 1]; ++t) gt += gpk[a.tie_slot[t]];
-        if (k == a.res_param) {
-            // d loglik / d f = (d loglik / d ln f) / f, summed over the contrasts
-            const double f = a.lo[k] + (a.hi[k] - a.lo[k]) * s;
-            double gr = 0.0;
-            for (int i = 0; i < a.n_contrast; ++i) gr += a.gres[(int64_t)c * a.n_contrast + i];
-            gt += gr / f;
-        }
-        const double g = gt * (a.hi[k] - a.lo[k]) * s * (1.0 - s) + (1.0 - 2.0 * s);
+        const double g = cofit_pull_back(a, c, k, uk, lp);
         if (a.stage == kStageLogp) {
             if (a.grad_out) a.grad_out[(int64_t)c * P + k] = g;
             continue;

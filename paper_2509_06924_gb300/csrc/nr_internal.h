@@ -180,13 +180,24 @@ cudaError_t launch_cofit_gather(const double *u, int C, int P, int NS, const int
                                 double *dq_scale, cudaStream_t st);
 cudaError_t launch_cofit_stage(const CofitStageArgs &a, cudaStream_t st);
 // variational inference (nr_vi.cu)
+// the slots a sampled u fills, as cofit_gather: theta_k or the fixed value
+struct CofitGatherArgs {
+    int32_t NS, NC, res_param;  // packed slots per chain, its stacks, resolution scale's parameter (-1: none)
+    const int32_t *src;         // [NS] parameter of a slot, or -1
+    const double *val;          // [NS] its fixed value
+    const double *lo, *hi;      // [P] prior bounds
+    double *params;             // [C x NS]
+    double *dq_scale;           // [C x NC] (res_param >= 0)
+};
 // vi_sample advances the device iteration counter and writes the Adam bias
 // corrections 1 / (1 - beta1^t), 1 / (1 - beta2^t) to bias[0..1]
 cudaError_t launch_vi_sample(const double *phi, const double *eps, int R, int P, double *u, double *part,
-                             int32_t *t_dev, double beta1, double beta2, double *bias, cudaStream_t st);
-cudaError_t launch_vi_adam(double *phi, double *m, double *v, const double *eps, const double *g,
-                           const double *logp, const double *part, int R, int P, const double *bias, double lr,
-                           double beta1, double beta2, double eps_adam, double *elbo, cudaStream_t st);
+                             int32_t *t_dev, double beta1, double beta2, double *bias, const CofitGatherArgs &a,
+                             cudaStream_t st);
+// a: the restarts as chains (C, P, u, ll, gpk, tie_*, lo, hi, res_param, gres); g: [C x P] workspace
+cudaError_t launch_vi_adam(double *phi, double *m, double *v, const double *eps, double *g, const double *part,
+                           const double *bias, double lr, double beta1, double beta2, double eps_adam, double *elbo,
+                           const CofitStageArgs &a, cudaStream_t st);
 
 // Raw per-stack sums of the mixed gradient kernels, and the stride of a
 // chunk's partial-sum slot: [accD (n) | accUr (n+1) | accUi (n+1) |

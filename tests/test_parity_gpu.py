@@ -809,6 +809,59 @@ def test_vi_step_parity_and_graph_replay():
     ctx.close()
 
 
+# A restart is one block: the number of free parameters against its threads
+# (rows of L in passes of 32, eight lanes a row), the sampled resolution
+# scale, and more parameters than the block stages in shared memory (2048).
+# Bounds as in the test above.
+@pytest.mark.parametrize("case", ["res", "many"])
+def test_vi_step_blocks(case):
+    from oracle import hmc
+    R = 3
+    if case == "res":
+        ctx, smp, ref, u_c, rng = sampler_setup(R, seed=5, res=True)
+    else:
+        rng = np.random.default_rng(8)
+        n, NC = 12, 40
+        q = W.log_grid(10, 0.01, 0.2)
+        val = np.concatenate([rand_stack(rng, n, d_range=(20, 60)) for _ in range(NC)])
+        L = W.layout(n)
+        half = np.empty(4 * n + 6)
+        for k, w in (("d", 5.0), ("rho", 2e-7), ("iota", 0.0), ("sigma", 0.0), ("scale", 0.05), ("bkg", 1e-8)):
+            half[L[k]] = w
+        v = val.reshape(NC, -1)
+        half = np.where(half > 0, half, 0.2 * np.abs(v))         # iota, sigma stay positive
+        lo, hi = (v - half).ravel(), (v + half + np.where(half > 0, 0.0, 1e-9)).ravel()
+        m = oracle.model(n, v[0], q, (0.05 * q).astype(np.float32), 5)
+        f32 = lambda a: np.asarray(a, np.float32)
+        ref = hmc.Model([n] * NC, [0] * NC, np.arange(val.size), val, lo, hi, [0, q.size], q, f32(0.05 * q),
+                        f32(1.03 * m), f32(0.05 * m), 5)
+        ctx = nr.Context(n_quad=5)
+        dev32 = lambda a: torch.as_tensor(f32(a), device="cuda")
+        smp = nr.Sampler(ctx, R, ref.n_layers, ref.dataset, ref.q_off, dev32(ref.Q), dev32(ref.dQ), dev32(ref.Robs),
+                         dev32(ref.err), ref.slot_src, val, lo, hi)
+        u_c = 0.2 * rng.normal(size=(R, ref.P))
+    P = ref.P
+    assert case == "res" or P > 2048
+    i, j = np.tril_indices(P)
+    tri = np.where(i == j, np.log(0.1), 0.02 / np.sqrt(P) * rng.normal(size=(R, i.size)))
+    phi = np.concatenate([u_c, tri], axis=1)
+    eps = rng.normal(size=(R, P))
+    dev = lambda a: torch.as_tensor(a, device="cuda")
+    ph, m, v, t = dev(phi), dev(0.0 * phi), dev(0.0 * phi), dev(np.array([0], np.int32))
+    elbo = smp.vi_step(ph, m, v, t, dev(eps), lr=0.05).cpu().numpy()
+    assert ctx.device_status() == 0
+    m = m.cpu().numpy()
+    for r in range(R):
+        u = u_c[r] + np.bincount(i, np.where(i == j, np.exp(tri[r]), tri[r]) * eps[r][j], P)
+        lp, g = ref.logp_grad(u)
+        el = lp + 0.5 * eps[r] @ eps[r] + tri[r][i == j].sum() + 0.5 * P * np.log(2 * np.pi)
+        assert abs(elbo[r] - el) <= 1e-5 * abs(el)
+        grad = np.concatenate([-g, np.where(i == j, -g[i] * eps[r][i] * np.exp(tri[r]) - 1.0, -g[i] * eps[r][j])])
+        assert np.max(np.abs(m[r] - 0.1 * grad)) <= 1e-4 * np.max(np.abs(0.1 * grad))
+    smp.close()
+    ctx.close()
+
+
 @pytest.mark.parametrize("name,S", [("uneven", 40), ("thick_oxide", 64), ("oled_cofit", 6), ("film_1l", 48)])
 def test_autotuned_plan_keeps_parity(name, S):
     """nr_plan with autotune = 1 times the candidate launch shapes (paired or
