@@ -447,6 +447,24 @@ def test_host_memory_calls_match_device_calls():
     assert torch.equal(ctx.loglik(bd).cpu(), ctx.loglik(bh))
 
 
+def test_autograd_backward_of_mixed_layer_counts():
+    """Stacks of different layer counts take the general form of backward,
+    stacks of one count the broadcast; both weight every stack's gradient by
+    its own factor, expanded (stride 0) or not."""
+    for S in ("uneven", "oled_cofit"):
+        wl = W.make_workload(S, n_stacks=5)
+        ctx = nr.Context(n_quad=wl.n_quad)
+        b = nr.Batch.from_workload(wl)
+        _, g = ctx.loglik_grad(b)
+        per = torch.as_tensor(4 * wl.n_layers.astype(np.int64) + 6, device=g.device)
+        for w in (torch.linspace(0.5, 2.0, wl.n_stacks, dtype=torch.float64, device=g.device),
+                  torch.full((1,), 0.3, dtype=torch.float64, device=g.device).expand(wl.n_stacks)):
+            params = b.params.clone().requires_grad_(True)
+            (got,) = torch.autograd.grad(nr.loglik_autograd(params, ctx, b), params, grad_outputs=w)
+            torch.testing.assert_close(got, g * torch.repeat_interleave(w, per), rtol=0, atol=0)
+        ctx.close()
+
+
 def test_autograd_function_backward_is_the_exact_gradient():
     wl = W.make_workload("film_1l", n_stacks=12)
     ctx = nr.Context(n_quad=wl.n_quad)
