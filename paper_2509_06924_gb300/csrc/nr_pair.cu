@@ -159,6 +159,20 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
     const int qs_end = wloc ? qs0 + tqw : TQ;
     const int nslots = (63 + K - 1) / K + 1;
     const int sgl = nslots <= 1 ? 32 : nslots <= 2 ? 16 : nslots <= 4 ? 8 : nslots <= 8 ? 4 : nslots <= 16 ? 2 : 1;
+    // per-thread places of the tile: staged Q point, w R entry, whether it leads
+    // its Q point, the row this lane adds up and the lanes that end with its sums
+    const int sg = lane / sgl, part = lane - sg * sgl;
+    const bool row_on = qs0 + sg < qs_end;
+    const int row_at = row_on ? (qs0 + sg) * KP : 0;
+    int slot_at[2], wr_at[2], from[2];
+    bool lead[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        slot_at[h] = lane_on[h] ? qslot[h] : 0;
+        wr_at[h] = qslot[h] * KP + kn[h];
+        lead[h] = lane_on[h] && kn[h] == 0;
+        from[h] = ((qslot[h] - qs0) * sgl) & 31;
+    }
     const float g_max = fmaxf(fabsf(qc.g_hi[0]), fabsf(qc.g_hi[K - 1]));
 
     for (int i = tid; i < 2 * WRN; i += BLOCK) (&sh_wR[0][0])[i] = 0.f; // padding stays 0
@@ -226,7 +240,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
         const float fsc = ka.dq_scale ? (float)ka.dq_scale[wi.stack] : 1.f; // resolution scale of the stack
         const float *rop = ka.r_obs + si.q_begin, *rep = ka.r_err + si.q_begin;
         const int span = (CAPQ / TQ) * TQ;
-        int sb = wi.q_lo, s_next = wi.q_lo, s_cnt = 0;
+        int sb = wi.q_lo, s_cnt = 0;
         auto consume = [&](int i) __attribute__((always_inline)) {
             if constexpr (LIK) {
                 const float2 rs = sh_rs[i];
@@ -274,7 +288,6 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                 sh_qd[i] = v;
             }
             sb = q0;
-            s_next = q0 + span;
             s_cnt = min(span, wi.q_hi - q0);
             __syncthreads();
         };
@@ -283,18 +296,13 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
         const float scale = sm.scale, bkg = sm.bkg;
         const f2 wks = pmul(wk, bc(scale));
         int buf = 0;
-        for (int q0 = wi.q_lo; q0 < wi.q_hi; q0 += TQ, buf ^= 1) {
-            if (q0 == s_next) restage(q0);
-            int qi[2], si_q[2];
-            bool act[2];
-            float4 qd[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                qi[h] = q0 + qslot[h];
-                si_q[h] = q0 - sb + (lane_on[h] ? qslot[h] : 0);
-                act[h] = lane_on[h] && qi[h] < wi.q_hi;
-                qd[h] = sh_qd[si_q[h]];
-            }
+        // t0: the tile's first Q point within the staged super-tile.  Slots past
+        // the last Q point are staged harmless (1/err = 0), so the tile needs no
+        // test of its end; idle lanes repeat slot 0 with weight 0.
+        for (int q0 = wi.q_lo; q0 < wi.q_hi; q0 += span) {
+        restage(q0);
+        for (int t0 = 0; t0 < s_cnt; t0 += TQ, buf ^= 1) {
+            const float4 qd[2] = {sh_qd[t0 + slot_at[0]], sh_qd[t0 + slot_at[1]]};
             const f2 Qh = make_float2(qd[0].x, qd[1].x), dQh = make_float2(qd[0].y, qd[1].y);
             // a1: node position k_0 = q/2 in double-float, k_0^2
             f2 k0h, k0l;
@@ -308,7 +316,6 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                 fast_two_sum2(s, e, k0h, k0l);
             }
             const b2 qok{k0h.x > 0.f, k0h.y > 0.f};
-            if ((act[0] && !qok.x) || (act[1] && !qok.y)) atomicOr(ka.status, NR_FLAG_BAD_Q);
             const f2 p_hi = pmul(k0h, k0h);
             f2 p_lo = pfma(k0h, k0h, pneg(p_hi));
             p_lo = pfma(padd(k0h, k0h), k0l, p_lo);
@@ -388,22 +395,23 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             } else {
                 R = pmul(pfma(B.re, B.re, pmul(B.im, B.im)), prcp(pfma(A.re, A.re, pmul(A.im, A.im))));
             }
-            if (!qok.x) R.x = __int_as_float(0x7fffffff);
-            if (!qok.y) R.y = __int_as_float(0x7fffffff);
+            if (!(qok.x && qok.y)) {
+                atomicOr(ka.status, NR_FLAG_BAD_Q);
+                if (!qok.x) R.x = __int_as_float(0x7fffffff);
+                if (!qok.y) R.y = __int_as_float(0x7fffffff);
+            }
 
             // a8-a10: smearing sum, model, residual, adjoint seed
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                if (lane_on[h]) sh_wR[buf][qslot[h] * KP + kn[h]] = half(wk, h) * half(R, h);
+                if (lane_on[h]) sh_wR[buf][wr_at[h]] = half(wk, h) * half(R, h);
             if (wloc) __syncwarp();
             else __syncthreads();
             f2 S;
             {
-                const int g = lane / sgl, part = lane - g * sgl;
-                const int slot = qs0 + g;
                 float ps = 0.f;
-                if (slot < qs_end) {
-                    const float4 *row = reinterpret_cast<const float4 *>(&sh_wR[buf][slot * KP]);
+                if (row_on) {
+                    const float4 *row = reinterpret_cast<const float4 *>(&sh_wR[buf][row_at]);
                     auto add4 = [&](int c) __attribute__((always_inline)) {
                         const float4 v = row[c];
                         ps += (v.x + v.y) + (v.z + v.w);
@@ -420,19 +428,20 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     }
                 }
                 for (int o = 1; o < sgl; o <<= 1) ps += __shfl_xor_sync(kFull, ps, o);
-                S.x = __shfl_sync(kFull, ps, ((qslot[0] - qs0) * sgl) & 31);
-                S.y = __shfl_sync(kFull, ps, ((qslot[1] - qs0) * sgl) & 31);
+                S.x = __shfl_sync(kFull, ps, from[0]);
+                S.y = __shfl_sync(kFull, ps, from[1]);
             }
             if constexpr (MODE == kModel) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    if (act[h] && kn[h] == 0) ka.r_out[si.out_off + qi[h]] = fmaf(scale, half(S, h), bkg);
+                    if (lead[h] && t0 + slot_at[h] < s_cnt)
+                        ka.r_out[si.out_off + sb + t0 + slot_at[h]] = fmaf(scale, half(S, h), bkg);
             } else {
                 const f2 ie = make_float2(fabsf(qd[0].w), fabsf(qd[1].w));
                 const f2 res = pmul(psub(pfma(bc(scale), S, bc(bkg)), make_float2(qd[0].z, qd[1].z)), ie);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    if (act[h] && kn[h] == 0) sh_rs[si_q[h]] = make_float2(half(res, h), half(S, h));
+                    if (lead[h]) sh_rs[t0 + slot_at[h]] = make_float2(half(res, h), half(S, h));
                 if constexpr (GRAD) {
                     const f2 Rb = pmul(wks, pneg(pmul(res, ie))); // w_k scale dl/dm (0 on idle slots)
 
@@ -448,6 +457,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     c2 kbar = czero();
                     Kz2 kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
                     c2 Xb_up = czero(); // Xbar_{j-1} (edge sweeps)
+                    const bool reach[2] = {lane_on[0] && qd[0].w < 0.f, lane_on[1] && qd[1].w < 0.f};
                     Kz2 kjm1 = kj;
                     const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
                     const f2 wres = RES ? pmul(dQh, g_hi) : bc(0.f);
@@ -492,7 +502,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                             b2 edge{false, false};
                             if constexpr (decltype(EDG)::value) {
                                 const f2 far = pmul(edge_u, kj.y); // |k_j|^2 < edge_u
-                                edge = b2{act[0] && far.x > 1.f, act[1] && far.y > 1.f};
+                                edge = b2{reach[0] && far.x > 1.f, reach[1] && far.y > 1.f};
 #pragma unroll
                                 for (int h = 0; h < 2; ++h) {
                                     const bool eh = h ? edge.y : edge.x;
@@ -553,13 +563,14 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     };
                     // the staged sign of 1/err marks Q points whose nodes may reach an
                     // interior-edge band (warp-uniform choice)
-                    if (__any_sync(kFull, (act[0] && qd[0].w < 0.f) || (act[1] && qd[1].w < 0.f)))
+                    if (__any_sync(kFull, reach[0] || reach[1]))
                         sweep(std::true_type{});
                     else
                         sweep(std::false_type{});
                     if constexpr (RES) gres_acc = pfma(wres, pfma(k0h, res_sum, res_k0), gres_acc);
                 } // GRAD
             } // LIK
+        }
         }
 
         if (tid == 0) sh_item = gridDim.x + atomicAdd(&ka.ticket[0], 1); // its latency overlaps the reductions

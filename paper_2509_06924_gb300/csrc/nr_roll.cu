@@ -211,6 +211,20 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
     const int qs_end = wloc ? qs0 + tqw : TQ;
     const int nslots = (63 + K - 1) / K + 1;
     const int sgl = nslots <= 1 ? 32 : nslots <= 2 ? 16 : nslots <= 4 ? 8 : nslots <= 8 ? 4 : nslots <= 16 ? 2 : 1;
+    // per-thread places of the tile: staged Q point, w R entry, whether it leads
+    // its Q point, the row this lane adds up and the lanes that end with its sums
+    const int sg = lane / sgl, part = lane - sg * sgl;
+    const bool row_on = qs0 + sg < qs_end;
+    const int row_at = row_on ? (qs0 + sg) * KP : 0;
+    int slot_at[2], wr_at[2], from[2];
+    bool lead[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        slot_at[h] = lane_on[h] ? qslot[h] : 0;
+        wr_at[h] = qslot[h] * KP + kn[h];
+        lead[h] = lane_on[h] && kn[h] == 0;
+        from[h] = ((qslot[h] - qs0) * sgl) & 31;
+    }
     const float g_max = fmaxf(fabsf(qc.g_hi[0]), fabsf(qc.g_hi[K - 1]));
 
     // the first items go round the SMs, one team each, the rest by ticket
@@ -263,7 +277,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         const float fsc = ka.dq_scale ? (float)ka.dq_scale[wi.stack] : 1.f; // resolution scale of the stack
         const float *rop = ka.r_obs + si.q_begin, *rep = ka.r_err + si.q_begin;
         const int span = (TS::CAPQ / TQ) * TQ;
-        int sb = wi.q_lo, s_next = wi.q_lo, s_cnt = 0;
+        int sb = wi.q_lo, s_cnt = 0;
         auto consume = [&](int i) __attribute__((always_inline)) {
             const float2 rs = ts.rs[i];
             const float Re = __ldg(rep + sb + i);
@@ -303,7 +317,6 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 ts.qd[i] = v;
             }
             sb = q0;
-            s_next = q0 + span;
             s_cnt = min(span, wi.q_hi - q0);
             team_sync(team);
         };
@@ -313,18 +326,13 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         const bool nc_big = sm.nc_big != 0;
         const f2 wks = pmul(wk, bc(scale));
         int buf = 0;
-        for (int q0 = wi.q_lo; q0 < wi.q_hi; q0 += TQ, buf ^= 1) {
-            if (q0 == s_next) restage(q0);
-            int qi[2], si_q[2];
-            bool act[2];
-            float4 qd[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                qi[h] = q0 + qslot[h];
-                si_q[h] = q0 - sb + (lane_on[h] ? qslot[h] : 0);
-                act[h] = lane_on[h] && qi[h] < wi.q_hi;
-                qd[h] = ts.qd[si_q[h]];
-            }
+        // t0: the tile's first Q point within the staged super-tile.  Slots past
+        // the last Q point are staged harmless (1/err = 0), so the tile needs no
+        // test of its end; idle lanes repeat slot 0 with weight 0.
+        for (int q0 = wi.q_lo; q0 < wi.q_hi; q0 += span) {
+        restage(q0);
+        for (int t0 = 0; t0 < s_cnt; t0 += TQ, buf ^= 1) {
+            const float4 qd[2] = {ts.qd[t0 + slot_at[0]], ts.qd[t0 + slot_at[1]]};
             const f2 Qh = make_float2(qd[0].x, qd[1].x), dQh = make_float2(qd[0].y, qd[1].y);
             // a1: node position k_0 = q/2 in double-float, k_0^2
             f2 k0h, k0l;
@@ -338,7 +346,6 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 fast_two_sum2(s, e, k0h, k0l);
             }
             const b2 qok{k0h.x > 0.f, k0h.y > 0.f};
-            if ((act[0] && !qok.x) || (act[1] && !qok.y)) atomicOr(ka.status, NR_FLAG_BAD_Q);
             const f2 p_hi = pmul(k0h, k0h);
             f2 p_lo = pfma(k0h, k0h, pneg(p_hi));
             p_lo = pfma(padd(k0h, k0h), k0l, p_lo);
@@ -384,37 +391,38 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             const c2 iA = cinv2(A); // 1 / A_0
             const c2 X0 = cmul2(B, iA);
             f2 R = pfma(X0.re, X0.re, pmul(X0.im, X0.im));
-            if (!qok.x) R.x = __int_as_float(0x7fffffff);
-            if (!qok.y) R.y = __int_as_float(0x7fffffff);
+            if (!(qok.x && qok.y)) {
+                atomicOr(ka.status, NR_FLAG_BAD_Q);
+                if (!qok.x) R.x = __int_as_float(0x7fffffff);
+                if (!qok.y) R.y = __int_as_float(0x7fffffff);
+            }
             tmem_wait_store();
 
             // a8-a10: smearing sum, model, residual, adjoint seed
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                if (lane_on[h]) ts.wR[buf][qslot[h] * KP + kn[h]] = half(wk, h) * half(R, h);
+                if (lane_on[h]) ts.wR[buf][wr_at[h]] = half(wk, h) * half(R, h);
             if (wloc) __syncwarp();
             else team_sync(team);
             f2 S;
             {
-                const int g = lane / sgl, part = lane - g * sgl;
-                const int slot = qs0 + g;
                 float ps = 0.f;
-                if (slot < qs_end) {
-                    const float4 *row = reinterpret_cast<const float4 *>(&ts.wR[buf][slot * KP]);
+                if (row_on) {
+                    const float4 *row = reinterpret_cast<const float4 *>(&ts.wR[buf][row_at]);
                     for (int c = part; c < KP / 4; c += sgl) {
                         const float4 v = row[c];
                         ps += (v.x + v.y) + (v.z + v.w);
                     }
                 }
                 for (int o = 1; o < sgl; o <<= 1) ps += __shfl_xor_sync(kFull, ps, o);
-                S.x = __shfl_sync(kFull, ps, ((qslot[0] - qs0) * sgl) & 31);
-                S.y = __shfl_sync(kFull, ps, ((qslot[1] - qs0) * sgl) & 31);
+                S.x = __shfl_sync(kFull, ps, from[0]);
+                S.y = __shfl_sync(kFull, ps, from[1]);
             }
             const f2 ie = make_float2(fabsf(qd[0].w), fabsf(qd[1].w));
             const f2 res = pmul(psub(pfma(bc(scale), S, bc(bkg)), make_float2(qd[0].z, qd[1].z)), ie);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                if (act[h] && kn[h] == 0) ts.rs[si_q[h]] = make_float2(half(res, h), half(S, h));
+                if (lead[h]) ts.rs[t0 + slot_at[h]] = make_float2(half(res, h), half(S, h));
             const f2 Rb = pmul(wks, pneg(pmul(res, ie))); // w_k scale dl/dm (0 on idle slots)
 
             // a7: adjoint sweep from the fronting down to the backing.  With
@@ -430,6 +438,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             c2 kj = c2{k0h, bc(0.f)};
             f2 yj = bc(0.f); // 1 / |k_j|^2
             c2 Xb_up = czero(); // Xbar_{j-1} (edge sweeps)
+            const bool reach[2] = {lane_on[0] && qd[0].w < 0.f, lane_on[1] && qd[1].w < 0.f};
             const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
             const f2 wres = RES ? pmul(dQh, g_hi) : bc(0.f);
             f2 res_sum = bc(0.f), res_k0 = bc(0.f);
@@ -485,7 +494,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     f2 inv = yj;
                     if constexpr (edg) {
                         const f2 far = pmul(edge_u, yj); // |k_j|^2 < edge_u
-                        const b2 edge{act[0] && far.x > 1.f, act[1] && far.y > 1.f};
+                        const b2 edge{reach[0] && far.x > 1.f, reach[1] && far.y > 1.f};
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const bool eh = h ? edge.y : edge.x;
@@ -537,9 +546,10 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             };
             // the staged sign of 1/err marks Q points whose nodes may reach an
             // interior-edge band (warp-uniform choice)
-            if (__any_sync(kFull, (act[0] && qd[0].w < 0.f) || (act[1] && qd[1].w < 0.f))) sweep(std::true_type{});
+            if (__any_sync(kFull, reach[0] || reach[1])) sweep(std::true_type{});
             else sweep(std::false_type{});
             if constexpr (RES) gres_acc = pfma(wres, pfma(k0h, res_sum, res_k0), gres_acc);
+        }
         }
         if (tid == 0) ts.item = workers + atomicAdd(&ka.ticket[0], 1); // its latency overlaps the reductions
         if (eq_cnt > 0) eq_drain();
