@@ -25,9 +25,17 @@ constexpr float kNcSmall = 0.125f;
 constexpr float kLog2Pi = 1.83787706640934548356f;       // ln(2 pi)
 constexpr unsigned kFull = 0xffffffffu;
 
-// |k_j|^2 < kEdgeFrac k_0^2 selects the interior-edge treatment of the adjoint
+// |k_j|^2 < kEdgeFrac k_0^2 selects the interior-edge treatment of the adjoint.
+// Outside the band the plain adjoint loses about k_0^2 / |k_j|^2 roundings of an
+// evaluation's own term, on an ever smaller share of the evaluations.  Bands
+// of 0.04, 0.02, 0.01 and 0.005 give the same errors against the oracle on
+// 200 ten-layer chains (median 3.5e-7, 99 % within 2.7e-6), 60 twelve-layer
+// ones (8.1e-7, 7.2e-6), 1500 thick films (2.2e-7, 2.1e-6), 1024 thin films and
+// 400 uneven stacks; a band of 0.01 queues a quarter of 0.04's entries:
+// twelve-layer gradients 26.2 -> 25.4 ms (49152 stacks), ten-layer 3.51 ->
+// 3.38 ms, 21-64 layers 1.78 -> 1.67 ms.
 #ifndef NR_EDGE_FRAC
-#define NR_EDGE_FRAC 0.04f
+#define NR_EDGE_FRAC 0.01f
 #endif
 constexpr float kEdgeFrac = NR_EDGE_FRAC;
 
