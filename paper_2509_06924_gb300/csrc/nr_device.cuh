@@ -486,7 +486,8 @@ struct StackSmem {
     float4 adj[NM + 1]; // interface j = 0..n: the adjoint's constants Re(s_j conj(N_j)) + 2 and - 2,
                         // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
     float scale, bkg;
-    int nc_big;         // 1: some interface's Nevot-Croce phase may exceed kNcSmall (cleared by the item's owner)
+    int nc_big[2];      // 1: some interface's Nevot-Croce phase may exceed kNcSmall (cleared by the item's
+                        // owner; two, so that an item can clear the next one's)
 };
 
 __device__ __forceinline__ float2 split_double(double v)
@@ -504,7 +505,7 @@ __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v
 // than one FP32 rounding of the parameter: with 48 such instructions a stack
 // here and 70 in the reductions, an item cost 0.8 us of its SM.
 template <int NM>
-__device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, int32_t *status)
+__device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int n, int tid, int32_t *status)
 {
     const int j = tid, lane = tid & 31;
     if (tid - lane > n + 1) return;
@@ -539,7 +540,7 @@ __device__ void stage_stack(StackSmem<NM> &sm, const double *p, int n, int tid, 
         // + 2 a a'; for |u| > 4 m of one sign it is below (0.6 (a + a'))^2 x 2
         const float D = fabsf(Nr), a = fmaxf(fabsf(aj), fabsf(adn));
         const float bound = -s * (0.5f * D + sqrtf(5.f * fmaxf(D, a) * a) + 1.2f * a);
-        if (!(bound <= kNcSmall)) sm.nc_big = 1; // every writer stores the same value
+        if (!(bound <= kNcSmall)) *nc_big = 1; // every writer stores the same value
     }
     if (j == 0) {
         const double scale = p[4 * n + 4], bkg = p[4 * n + 5];

@@ -232,7 +232,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
     int item = team * gridDim.x + blockIdx.x;
     for (; item < ka.n_items;) {
         const WorkItem wi = ka.items[item];
-        if (tid == 0) sm.nc_big = 0;
+        if (tid == 0) sm.nc_big[0] = 0;
         team_sync(team);
         if constexpr (NR_DEBUG) {
             if (!item_in_bounds(ka, wi, NMAX)) { // uniform over the team
@@ -249,7 +249,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         const StackInfo si = ka.stacks[wi.stack];
         const int n = si.n;
         const double *p = ka.params + si.par_off;
-        stage_stack<NM>(sm, p, n, tid, ka.status);
+        stage_stack<NM>(sm, &sm.nc_big[0], p, n, tid, ka.status);
         for (int i = lane; i < (n + 2) * 32; i += 32) acc[i] = 0.f;
 
         // step j's four sums: over the quad's lanes, one sum left in each lane
@@ -323,7 +323,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         team_sync(team);
 
         const float scale = sm.scale, bkg = sm.bkg;
-        const bool nc_big = sm.nc_big != 0;
+        const bool nc_big = sm.nc_big[0] != 0;
         const f2 wks = pmul(wk, bc(scale));
         int buf = 0;
         // t0: the tile's first Q point within the staged super-tile.  Slots past
