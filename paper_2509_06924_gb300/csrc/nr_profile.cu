@@ -20,7 +20,7 @@
 // and only the interfaces that a ballot names are evaluated, each as its
 // difference from what the base already counts.  That holds for any order of
 // the depths (a run then just spans more).  16384 stacks of ten layers x 512
-// depths, both curves: 165 -> 51 us a call (1.4 TB/s of its 67 MB output and
+// depths, both curves: 165 -> 45 us a call (1.6 TB/s of its 67 MB output and
 // parameters; stacks of one layer count upload no metadata either).
 //
 // A CTA stages 8 stacks at a time, one per warp: lane j forms interface j's
@@ -60,6 +60,9 @@ __device__ __forceinline__ int float_order(float x)
 }
 __device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
 
+// finite, by the exponent bits (an FP64 comparison of a warp takes 16 cycles of its SM)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
 // One warp stages stack parameters p (n layers) into st.
 __device__ void stage_profile(ProfileStack &st, const double *p, int n, int lane, int32_t *status)
 {
@@ -94,14 +97,15 @@ __device__ void stage_profile(ProfileStack &st, const double *p, int n, int lane
         if (on) {
             const double rj = p[n + j], rj1 = p[n + j + 1];
             const double ij = j >= 1 ? p[2 * n + 2 + j - 1] : 0.0, ij1 = p[2 * n + 2 + j];
-            const float sg = (float)p[3 * n + 3 + j];
+            const double sgd = p[3 * n + 3 + j];
+            const float sg = (float)sgd;
             st.at[j] = make_float4(h, l, sg > 0.f ? 1.f / (1.41421356237f * sg) : 0.f, (float)(rj1 - rj));
             // a little past 4 sqrt(2) sigma, and past the rounding of z - z_j
             const float reach = fmaf(1.41421356237f * 1.00001f * kErfOne, fmaxf(sg, 0.f), 1e-6f * fabsf(h) + 1e-30f);
             st.med[j] = make_float4((float)(ij1 - ij), reach, (float)rj1, (float)ij1);
             if (j == 0) st.rho0 = (float)rj;
-            bad |= !isfinite(d) || !isfinite(rj) || !isfinite(rj1) || !isfinite(ij) || !isfinite(ij1) ||
-                   !isfinite(sg) || sg < 0.f;
+            bad |= !finite_bits(d) || !finite_bits(rj) || !finite_bits(rj1) || !finite_bits(ij) ||
+                   !finite_bits(ij1) || !finite_bits(sgd) || sg < 0.f;
         }
     }
     bad = __any_sync(kAll, bad);
@@ -126,19 +130,33 @@ nr_profile_kernel(const double *params, const int64_t *par_off, const int32_t *n
         }
         __syncthreads();
         const int here = min(kProfileWarps, n_stacks - s0);
-        for (int64_t pair = warp; pair < (int64_t)here * runs; pair += kProfileWarps) {
-            const int k = (int)(pair / runs);
-            const int q0 = (int)(pair - (int64_t)k * runs) * kRun;
+        // the 8 stacks' runs, run by run, in equal shares: a warp forms a run's
+        // span once for the stacks it takes it for
+        const int total = here * runs, share = (total + kProfileWarps - 1) / kProfileWarps;
+        int at = warp * share;
+        const int end = min(at + share, total);
+        int run = at / here, k = at - run * here;
+        float z0 = 0.f, z1 = 0.f, zlo = 0.f, zhi = 0.f, slack = 0.f;
+        for (bool fresh = true; at < end; ++at, ++k) {
+            if (k == here) {
+                k = 0;
+                ++run;
+                fresh = true;
+            }
+            const int i0 = run * kRun + lane, i1 = i0 + 32;
+            if (fresh) {
+                fresh = false;
+                z0 = z[min(i0, nz - 1)];
+                z1 = z[min(i1, nz - 1)];
+                // the run's span; a NaN depth or parameter evaluates everything
+                const int o0 = float_order(z0), o1 = float_order(z1);
+                zlo = order_float(__reduce_min_sync(kAll, min(o0, o1)));
+                zhi = order_float(__reduce_max_sync(kAll, max(o0, o1)));
+                slack = 1e-6f * fmaxf(fabsf(zlo), fabsf(zhi)); // rounding of z - z_j
+            }
             const ProfileStack &st = sh[k];
             const int n = st.n >= 0 ? st.n : -1 - st.n;
-            const int i0 = q0 + lane, i1 = i0 + 32;
-            const float z0 = z[min(i0, nz - 1)], z1 = z[min(i1, nz - 1)];
-            // the run's span; a NaN depth or parameter evaluates everything
-            const int o0 = float_order(z0), o1 = float_order(z1);
-            const float zlo = order_float(__reduce_min_sync(kAll, min(o0, o1)));
-            const float zhi = order_float(__reduce_max_sync(kAll, max(o0, o1)));
             const bool plain = st.n >= 0 && zhi - zlo >= 0.f;
-            const float slack = 1e-6f * fmaxf(fabsf(zlo), fabsf(zhi)); // rounding of z - z_j
             unsigned above[kRounds], eval[kRounds]; // interfaces wholly above the run; those to evaluate
             int m = 0;                              // the base counts interfaces 0 .. m-1 whole
 #pragma unroll
