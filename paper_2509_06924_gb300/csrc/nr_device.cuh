@@ -486,6 +486,7 @@ struct StackSmem {
     float4 adj[NM + 1]; // interface j = 0..n: the adjoint's constants Re(s_j conj(N_j)) + 2 and - 2,
                         // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
     float scale, bkg;
+    int p_max;          // bits of the largest k_0^2 or |c_j| of the item so far (split_media)
     int nc_big[2];      // 1: some interface's Nevot-Croce phase may exceed kNcSmall (cleared by the item's
                         // owner; two, so that an item can clear the next one's)
 };
@@ -549,6 +550,36 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
         bad |= !finite_bits(scale) || !finite_bits(bkg);
     }
     if (bad) atomicOr(status, NR_FLAG_NONFINITE_PARAM);
+}
+
+// Common quantum.  k_0^2 - c_j needs both words of both operands (the layer
+// phase), and an error-free difference of the high words costs six
+// operations per layer.  With every high word a multiple of one quantum g and
+// below 2^23 g, the plain difference is exact, and the low words (at most
+// g / 2) make up the rest to 2^-47 of the largest operand.  The kernels whose
+// sweeps are loops over many layers split k_0^2 and the c_j that way, with g
+// from the largest k_0^2 of the Q points staged so far and the largest |c_j|:
+// x + M - M rounds x to a multiple of g, M = 1.5 x 2^23 g.
+// 10000 stacks of 1-20 layers, log-likelihood 1.523 -> 1.439 ms; ten-layer
+// model curves 1.550 -> 1.494 ms; gradients 0.5-1.4 % faster; errors unchanged.
+// One and two layers do not repay the split itself.
+__device__ __forceinline__ int quantum_bits(float v) { return v < 1e30f ? __float_as_int(v) : 0; } // v >= 0; not NaN
+__device__ __forceinline__ float quantum_magic(int p_max)
+{
+    return __int_as_float(((p_max >> 23) + 3) << 23 | 0x400000); // 2^22 g at least twice the maximum
+}
+// thread j - 1 splits medium j again; between barriers
+template <int NM>
+__device__ __forceinline__ void split_media(StackSmem<NM> &sm, int n, int tid, float M)
+{
+    if (tid <= n) {
+        float4 m = sm.med[tid + 1];
+        const float c = m.x + m.y;
+        const float h = __fadd_rn(__fadd_rn(c, M), -M);
+        m.y = __fadd_rn(__fadd_rn(m.x, -h), m.y);
+        m.x = h;
+        sm.med[tid + 1] = m;
+    }
 }
 
 // v0 + v1 + v2 + v3 (+ lo) to FP64 accuracy of the floats' sum: error-free

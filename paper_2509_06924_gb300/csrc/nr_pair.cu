@@ -98,6 +98,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
     constexpr int BLOCK = kPairBlock;
     constexpr int WARPS = BLOCK / 32;
     constexpr bool RES = MODE == kGradRes;
+    constexpr bool QUANT = PT::RFWD; // wavevectors from a common quantum (split_media)
     constexpr int NACC = PT::NACC;
     constexpr int NRAW = 4 * NM + 7;
     constexpr int CAPQ = 256;
@@ -279,11 +280,17 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             }
             return v;
         };
+        int p_bits = 0; // largest k_0^2 (or |c_j|) this thread staged (QUANT)
+        float magic = 0.f;
         auto place = [&](int i, int qa, float4 r) __attribute__((always_inline)) {
             float4 v = make_float4(0.05f, 0.f, 0.f, 0.f); // past the end: a harmless node, 1/err = 0
             if (qa < wi.q_hi) {
                 v.x = 0.5f * r.x;
                 v.y = 0.5f * fsc * r.y;
+                if constexpr (QUANT) {
+                    const float k = fabsf(v.x) + fabsf(v.y) * g_max;
+                    p_bits = max(p_bits, quantum_bits(k * k));
+                }
                 if constexpr (LIK) {
                     v.z = r.z;
                     v.w = rcp_approx(r.w);
@@ -313,6 +320,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             first1 = fetch(wi.q_lo + tid + BLOCK);
         }
         stage_stack<NM>(sm, &sm.nc_big[par], p, n, tid, ka.status);
+        if (QUANT && tid == 0) sm.p_max = 0;
         __syncthreads();
         if (tid == 0) sm.nc_big[par ^ 1] = 0;
         auto restage = [&](int q0) {
@@ -328,6 +336,14 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             }
             sb = q0;
             s_cnt = min(span, wi.q_hi - q0);
+            if constexpr (QUANT) {
+                if (tid <= n) p_bits = max(p_bits, quantum_bits(fabsf(sm.med[tid + 1].x + sm.med[tid + 1].y)));
+                p_bits = __reduce_max_sync(kFull, p_bits);
+                if (lane == 0) atomicMax(&sm.p_max, p_bits);
+                __syncthreads();
+                magic = quantum_magic(sm.p_max);
+                split_media(sm, n, tid, magic);
+            }
             __syncthreads();
         };
 
@@ -354,9 +370,10 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                 fast_two_sum2(s, e, k0h, k0l);
             }
             const b2 qok{k0h.x > 0.f, k0h.y > 0.f};
-            const f2 p_hi = pmul(k0h, k0h);
+            f2 p_hi = pmul(k0h, k0h);
             f2 p_lo = pfma(k0h, k0h, pneg(p_hi));
             p_lo = pfma(padd(k0h, k0h), k0l, p_lo);
+            if constexpr (QUANT) quantise2(p_hi, p_lo, magic);
 
             // a3-a6 forward from the backing up, projective (X_j = B_j / A_j);
             // the gradient kernels keep every intermediate
@@ -364,12 +381,12 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             Kz2 kst[NK];
             c2 rst[NK], Gst[NK], Est[NK], bst[NK], Ast[NK];
             c2 A = c2{bc(1.f), bc(0.f)}, B = czero();
-            Kz2 kbelow = medium_kz2<false>(p_hi, p_lo, sm.med[n + 1]);
+            Kz2 kbelow = medium_kz2<false, QUANT>(p_hi, p_lo, sm.med[n + 1]);
             auto fwd_step = [&](int j, auto TOP, auto BOT, auto TRIG) __attribute__((always_inline)) {
                 const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                 Kz2 kj;
-                if (top) kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
-                else kj = medium_kz2<true>(p_hi, p_lo, sm.med[j]);
+                if (top) kj = Kz2{k0h, bc(0.f), k0l, QUANT ? padd(p_hi, p_lo) : p_hi, bc(0.f)};
+                else kj = medium_kz2<true, QUANT>(p_hi, p_lo, sm.med[j]);
                 const float4 Ij = sm.itf[j];
                 const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs)
                                   : fresnel_g2<false, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs);

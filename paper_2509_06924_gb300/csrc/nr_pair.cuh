@@ -137,14 +137,28 @@ __device__ __forceinline__ Kz2 kz_sqrt2(f2 uh, f2 ul, float a, float a2)
     return k;
 }
 
-// k of medium j >= 1 from k_0^2 = (p_hi + p_lo) and the staged medium entry
-template <bool REFINE>
+// k_0^2 split by the quantum of magic number M
+__device__ __forceinline__ void quantise2(f2 &p_hi, f2 &p_lo, float M)
+{
+    const f2 h = padd(padd(p_hi, bc(M)), bc(-M));
+    p_lo = padd(psub(p_hi, h), p_lo);
+    p_hi = h;
+}
+
+// k of medium j >= 1 from k_0^2 = (p_hi + p_lo) and the staged medium entry;
+// QUANT: both split by a common quantum (split_media)
+template <bool REFINE, bool QUANT>
 __device__ __forceinline__ Kz2 medium_kz2(f2 p_hi, f2 p_lo, float4 m)
 {
     if constexpr (REFINE) {
         f2 uh, ul;
-        two_sum2(p_hi, bc(-m.x), uh, ul);
-        ul = padd(ul, padd(p_lo, bc(-m.y)));
+        if constexpr (QUANT) {
+            uh = padd(p_hi, bc(-m.x)); // exact
+            ul = padd(p_lo, bc(-m.y));
+        } else {
+            two_sum2(p_hi, bc(-m.x), uh, ul);
+            ul = padd(ul, padd(p_lo, bc(-m.y)));
+        }
         fast_two_sum2(uh, ul, uh, ul);
         return kz_sqrt2<true>(uh, ul, m.z, m.w);
     } else {

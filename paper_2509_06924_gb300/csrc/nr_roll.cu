@@ -232,7 +232,10 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
     int item = team * gridDim.x + blockIdx.x;
     for (; item < ka.n_items;) {
         const WorkItem wi = ka.items[item];
-        if (tid == 0) sm.nc_big[0] = 0;
+        if (tid == 0) {
+            sm.nc_big[0] = 0;
+            sm.p_max = 0;
+        }
         team_sync(team);
         if constexpr (NR_DEBUG) {
             if (!item_in_bounds(ka, wi, NMAX)) { // uniform over the team
@@ -290,7 +293,9 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             gsc_acc = fmaf(dldm, rs.y, gsc_acc);
             gbk_acc += dldm;
         };
+        float magic = 0.f; // of the common quantum (split_media)
         auto restage = [&](int q0) {
+            int p_bits = 0; // largest k_0^2 or |c_j| this thread sees
             team_sync(team); // the previous super-tile's reads and pairs are complete
             for (int i = tid; i < span; i += kTeam) {
                 if (i < s_cnt) consume(i);
@@ -305,11 +310,12 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     // (negative 1/err: yes)
                     const float a = fabsf(v.y) * g_max;
                     const float lo = fmaxf(v.x - a, 0.f), hi = v.x + a;
+                    p_bits = max(p_bits, quantum_bits(hi * hi));
                     const float k2lo = lo * lo * (1.f - 1.5f * kEdgeFrac);
                     const float k2hi = hi * hi * (1.f + 1.5f * kEdgeFrac);
                     bool e = false;
                     for (int j = 1; j <= n; ++j) {
-                        const float c = sm.med[j].x;
+                        const float c = sm.med[j].x + sm.med[j].y;
                         e |= c > 0.f && c < k2hi && c > k2lo;
                     }
                     if (e && v.w > 0.f) v.w = -v.w;
@@ -318,6 +324,12 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             }
             sb = q0;
             s_cnt = min(span, wi.q_hi - q0);
+            if (tid <= n) p_bits = max(p_bits, quantum_bits(fabsf(sm.med[tid + 1].x + sm.med[tid + 1].y)));
+            p_bits = __reduce_max_sync(kFull, p_bits);
+            if (lane == 0) atomicMax(&sm.p_max, p_bits);
+            team_sync(team);
+            magic = quantum_magic(sm.p_max);
+            split_media(sm, n, tid, magic);
             team_sync(team);
         };
         team_sync(team);
@@ -346,9 +358,10 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 fast_two_sum2(s, e, k0h, k0l);
             }
             const b2 qok{k0h.x > 0.f, k0h.y > 0.f};
-            const f2 p_hi = pmul(k0h, k0h);
+            f2 p_hi = pmul(k0h, k0h);
             f2 p_lo = pfma(k0h, k0h, pneg(p_hi));
             p_lo = pfma(padd(k0h, k0h), k0l, p_lo);
+            quantise2(p_hi, p_lo, magic);
             __syncwarp();
 
             // a3-a6 forward from the backing up (n >= 3: the top, middle and
@@ -356,9 +369,9 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             c2 A = c2{bc(1.f), bc(0.f)}, B;
             auto forward = [&](auto TRIG) __attribute__((always_inline)) {
                 constexpr int T = decltype(TRIG)::value;
-                Kz2 kb = medium_kz2<false>(p_hi, p_lo, sm.med[n + 1]);
+                Kz2 kb = medium_kz2<false, true>(p_hi, p_lo, sm.med[n + 1]);
                 {
-                    const Kz2 kj = medium_kz2<true>(p_hi, p_lo, sm.med[n]);
+                    const Kz2 kj = medium_kz2<true, true>(p_hi, p_lo, sm.med[n]);
                     const float4 I = sm.itf[n];
                     const c2 G = fresnel_g2<false, T>(kj, kb, I, sm.lay[n + 1].w, sh_cs);
                     B = cscl2(I.x, I.y, G);
@@ -368,8 +381,8 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 auto step = [&](int j, auto TOP) __attribute__((always_inline)) {
                     constexpr bool top = decltype(TOP)::value;
                     Kz2 kj;
-                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
-                    else kj = medium_kz2<true>(p_hi, p_lo, sm.med[j]);
+                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, padd(p_hi, p_lo), bc(0.f)};
+                    else kj = medium_kz2<true, true>(p_hi, p_lo, sm.med[j]);
                     const float4 I = sm.itf[j];
                     const float4 L = sm.lay[j + 1];
                     const c2 G = fresnel_g2<top, T>(kj, kb, I, L.w, sh_cs);
@@ -449,7 +462,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 Slot sl;
                 if constexpr (!bot) tmem_load(tm + j * kSlotCols, sl);
                 const float4 I = sm.itf[j], C = sm.adj[j];
-                const Kz2 kz1 = medium_kz2<false>(p_hi, p_lo, sm.med[j + 1]);
+                const Kz2 kz1 = medium_kz2<false, true>(p_hi, p_lo, sm.med[j + 1]);
                 const c2 kj1 = kc2(kz1);
                 const float4 bv = ts.b[(bot ? NM : j) * kTeam + tid];
                 c2 G, b = czero(), kbar1 = czero(), rb = Bb, Xb_in = czero();

@@ -360,6 +360,48 @@ def test_rolled_gradient_kernel_bucket_edges(K):
                  {"loglik": TOL_LL, "grad": TOL_G})
 
 
+# Sweeps over more than two layers (and the forward ones) take k_0^2 - c_j from
+# a common quantum that grows with the Q points staged so far: several
+# super-tiles in ascending and in shuffled order, Q up to 1.2 (the quantum far
+# above the low-Q nodes' own rounding), fronting media denser than the layers
+# (negative c_j), equal SLDs (c_j = 0) and a dense metal.  The bounds are the
+# module's.
+@pytest.mark.parametrize("order", ["up", "shuffled"])
+def test_common_quantum(order):
+    rng = np.random.default_rng(17)
+    q = np.concatenate([W.log_grid(180, 0.004, 1.2), W.log_grid(120, 0.008, 0.03)])
+    q = np.sort(q) if order == "up" else rng.permutation(q)
+    datasets = [(q, 0.04 * q.astype(np.float64))]
+    stacks = []
+    for n in (0, 3, 4, 9, 20, 33):
+        for front in (0.0, 6.35e-6):
+            st = rand_stack(rng, n, front=front, d_range=(10, 80) if n > 10 else (20, 400))
+            if n >= 3:
+                st[W.layout(n)["rho"]][1:3] = (front, 1.2e-5)
+            stacks.append((n, st, 0))
+    wl = custom_workload(stacks, datasets)
+    assert_parity(wl, run_gpu(wl), run_oracle(wl))
+
+
+def test_a_bad_q_point_leaves_the_others():
+    """A non-positive or NaN Q point raises the flag and spoils its own model
+    value only."""
+    rng = np.random.default_rng(18)
+    q = W.log_grid(90, 0.01, 0.2)
+    wl = custom_workload([(n, rand_stack(rng, n), 0) for n in (1, 2, 6, 24)], [(q, 0.03 * q.astype(np.float64))])
+    good = run_gpu(wl, modes=("model",))["m"].reshape(4, -1)
+    wl.q = wl.q.copy()
+    wl.q[[7, 40]] = (-0.01, np.nan)
+    ctx = nr.Context(n_quad=wl.n_quad)
+    m = ctx.reflectivity(nr.Batch.from_workload(wl)).cpu().numpy().astype(np.float64).reshape(4, -1)
+    assert ctx.device_status() & nr.NR_FLAG_BAD_Q
+    ctx.close()
+    keep = np.setdiff1d(np.arange(q.size), [7, 40])
+    assert np.all(np.isnan(m[:, [7, 40]])) and np.all(np.isfinite(m[:, keep]))
+    # the quantum may differ by the spoiled points: within the model bound
+    assert np.max(np.abs(np.log(m[:, keep]) - np.log(good[:, keep]))) <= TOL_M
+
+
 def test_zero_resolution_is_unsmeared():
     wl = W.make_workload("thick_oxide", n_stacks=16)
     wl.dq = np.zeros_like(wl.dq)
