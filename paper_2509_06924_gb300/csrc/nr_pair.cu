@@ -381,12 +381,12 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             Kz2 kst[NK];
             c2 rst[NK], Gst[NK], Est[NK], bst[NK], Ast[NK];
             c2 A = c2{bc(1.f), bc(0.f)}, B = czero();
-            Kz2 kbelow = medium_kz2<false, QUANT>(p_hi, p_lo, sm.med[n + 1]);
+            Kz2 kbelow = medium_kz2<kRootPlain, QUANT>(p_hi, p_lo, sm.med[n + 1]);
             auto fwd_step = [&](int j, auto TOP, auto BOT, auto TRIG) __attribute__((always_inline)) {
                 const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                 Kz2 kj;
                 if (top) kj = Kz2{k0h, bc(0.f), k0l, QUANT ? padd(p_hi, p_lo) : p_hi, bc(0.f)};
-                else kj = medium_kz2<true, QUANT>(p_hi, p_lo, sm.med[j]);
+                else kj = medium_kz2<TAB ? kRootFull : kRootPhase, QUANT>(p_hi, p_lo, sm.med[j]);
                 const float4 Ij = sm.itf[j];
                 const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs)
                                   : fresnel_g2<false, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs);

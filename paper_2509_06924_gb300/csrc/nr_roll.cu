@@ -369,9 +369,9 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             c2 A = c2{bc(1.f), bc(0.f)}, B;
             auto forward = [&](auto TRIG) __attribute__((always_inline)) {
                 constexpr int T = decltype(TRIG)::value;
-                Kz2 kb = medium_kz2<false, true>(p_hi, p_lo, sm.med[n + 1]);
+                Kz2 kb = medium_kz2<kRootPlain, true>(p_hi, p_lo, sm.med[n + 1]);
                 {
-                    const Kz2 kj = medium_kz2<true, true>(p_hi, p_lo, sm.med[n]);
+                    const Kz2 kj = medium_kz2<kRootFull, true>(p_hi, p_lo, sm.med[n]);
                     const float4 I = sm.itf[n];
                     const c2 G = fresnel_g2<false, T>(kj, kb, I, sm.lay[n + 1].w, sh_cs);
                     B = cscl2(I.x, I.y, G);
@@ -382,7 +382,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     constexpr bool top = decltype(TOP)::value;
                     Kz2 kj;
                     if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, padd(p_hi, p_lo), bc(0.f)};
-                    else kj = medium_kz2<true, true>(p_hi, p_lo, sm.med[j]);
+                    else kj = medium_kz2<kRootFull, true>(p_hi, p_lo, sm.med[j]);
                     const float4 I = sm.itf[j];
                     const float4 L = sm.lay[j + 1];
                     const c2 G = fresnel_g2<top, T>(kj, kb, I, L.w, sh_cs);
@@ -462,7 +462,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 Slot sl;
                 if constexpr (!bot) tmem_load(tm + j * kSlotCols, sl);
                 const float4 I = sm.itf[j], C = sm.adj[j];
-                const Kz2 kz1 = medium_kz2<false, true>(p_hi, p_lo, sm.med[j + 1]);
+                const Kz2 kz1 = medium_kz2<kRootPlain, true>(p_hi, p_lo, sm.med[j + 1]);
                 const c2 kj1 = kc2(kz1);
                 const float4 bv = ts.b[(bot ? NM : j) * kTeam + tid];
                 c2 G, b = czero(), kbar1 = czero(), rb = Bb, Xb_in = czero();
