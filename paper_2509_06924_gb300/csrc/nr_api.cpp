@@ -12,6 +12,7 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -360,28 +361,46 @@ std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std:
     int64_t nst = 0;
     double res_w = 0.0, w_sum = 0.0;
     std::vector<std::vector<ChunkCand>> cands(gs.size());
-    auto dlen = [&](int s) { return pl.q_off[pl.dataset[s] + 1] - pl.q_off[pl.dataset[s]]; };
-    auto cost_of = [&](const GroupSpan &g, int64_t chunk) {
+    // the stacks of a group by kind (layers and points): a batch has few
+    struct Kind {
+        int n;
+        int64_t len;
+        double count;
+    };
+    std::vector<std::vector<Kind>> kinds(gs.size());
+    auto cost_of = [&](size_t k, int64_t chunk) {
+        const GroupSpan &g = gs[k];
         const ItemCost ic = item_cost(mode, g.nmax);
         ChunkCand c{chunk, 0.0, 0.0, 0};
-        for (size_t i = g.i0; i < g.i1; ++i) {
-            const int s = order[i];
-            const int64_t len = std::max<int64_t>(dlen(s), 1), ch = std::min(chunk, len);
+        for (const Kind &kd : kinds[k]) {
+            const int64_t len = std::max<int64_t>(kd.len, 1), ch = std::min(chunk, len);
             const int64_t nch = (len + ch - 1) / ch, rest = len - (nch - 1) * ch;
-            const double w = ic.tile * (pl.n_layers[s] + 1.0);
+            const double w = ic.tile * (kd.n + 1.0);
             const int64_t t = (ch + g.tile_q - 1) / g.tile_q, tr = (rest + g.tile_q - 1) / g.tile_q;
-            c.total += w * (double)((nch - 1) * t + tr) + (double)nch * ic.item;
+            c.total += kd.count * (w * (double)((nch - 1) * t + tr) + (double)nch * ic.item);
             c.big = std::max(c.big, w * (double)t + ic.item);
-            c.items += nch;
+            c.items += (int64_t)kd.count * nch;
         }
         return c;
     };
+    auto dlen = [&](int s) { return pl.q_off[pl.dataset[s] + 1] - pl.q_off[pl.dataset[s]]; };
+    int64_t most = 0; // consumers of the largest launch
     for (size_t k = 0; k < gs.size(); ++k) {
-        int64_t max_len = 1;
-        for (size_t i = gs[k].i0; i < gs[k].i1; ++i) max_len = std::max(max_len, dlen(order[i]));
-        whole[k] = max_len;
         nst += (int64_t)(gs[k].i1 - gs[k].i0);
-        const ChunkCand w = cost_of(gs[k], max_len);
+        most = std::max(most, gs[k].resident);
+        for (size_t i = gs[k].i0; i < gs[k].i1; ++i) whole[k] = std::max(whole[k], dlen(order[i]));
+    }
+    if (nst >= kChunkWaves * most) return whole;
+    for (size_t k = 0; k < gs.size(); ++k) {
+        std::unordered_map<int64_t, size_t> at;
+        for (size_t i = gs[k].i0; i < gs[k].i1; ++i) {
+            const int s = order[i];
+            const int64_t len = dlen(s);
+            const auto found = at.try_emplace(len * (NR_MAX_LAYERS + 1) + pl.n_layers[s], kinds[k].size());
+            if (found.second) kinds[k].push_back(Kind{pl.n_layers[s], len, 0.0});
+            kinds[k][found.first->second].count += 1.0;
+        }
+        const ChunkCand w = cost_of(k, whole[k]);
         res_w += w.total * (double)gs[k].resident;
         w_sum += w.total;
         cands[k].push_back(w);
@@ -393,7 +412,7 @@ std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std:
         // chunk lengths of 1..16 tiles, then growing by a quarter (a few
         // dozen candidates however long the datasets are)
         for (int64_t mt = 1; mt * gs[k].tile_q < whole[k]; mt = mt < 16 ? mt + 1 : mt + (mt + 3) / 4)
-            cands[k].push_back(cost_of(gs[k], mt * gs[k].tile_q));
+            cands[k].push_back(cost_of(k, mt * gs[k].tile_q));
     // items of mean time `mean` and largest `big`, `n` of them: full rounds of
     // R at the full rate, then the last round at its own concurrency
     auto time_of = [&](double total, double big, double n) {
