@@ -65,9 +65,12 @@ CIS_NC = 20
 
 
 def flops_per_eval(n: int, K: int) -> float:
-    """Algorithmic FP32 flops of one fwd+grad evaluation of an n-layer stack
-    (FMA = 2), counted term by term from the gradient kernel's source,
-    including the FP32 arithmetic of the table-driven sin/cos.  Not counted:
+    """FP32 flops of one fwd+grad evaluation of an n-layer stack (FMA = 2) in
+    the Moebius form, counted term by term, including the FP32 arithmetic of
+    the table-driven sin/cos and, above two layers, of forming the factors
+    again in the adjoint: the yardstick every kernel is measured with.  The
+    kernels need fewer (projective form, factors kept); what they execute is
+    the lane operations that the profiles count.  Not counted:
     special-function (XU) operations, compares and selects, and the redundant
     copies of the smearing sum that every lane of a Q point forms."""
     store = n <= 2

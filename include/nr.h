@@ -97,7 +97,9 @@ typedef struct nr_options {
     int32_t autotune;      /* 1: nr_plan times launch shapes and caches them  */
     int32_t tile_q;        /* override: Q points per CTA tile (0 = auto)      */
     int32_t chunk_q;       /* override: Q points per work item (0 = auto)     */
-    int32_t grid_ctas;     /* override: persistent CTAs (0 = auto)            */
+    int32_t grid_ctas;     /* override: consumers of a launch's work queue
+                              (0 = auto): CTAs, or the 128-thread teams of
+                              the 3-and-more-layer gradients               */
     int32_t serial;        /* 1: launch the register buckets of a batch one
                               after another on the call's stream; 0 (default):
                               concurrently on forked streams joined back into
@@ -203,7 +205,8 @@ nr_status nr_device_status(nr_ctx *ctx, void *stream, int32_t *flags);
 nr_status nr_quadrature(int32_t K, double *x, double *w);
 
 /* Evaluations (stack x Q point x quadrature node) one compute call performs
- * on this batch, and the launch shape last chosen for it (for reporting).
+ * on this batch, and the launch shape last chosen for it (for reporting;
+ * grid_ctas: consumers of the work queue, as in nr_options).
  * Any output pointer may be NULL. */
 nr_status nr_plan_info(nr_ctx *ctx, const nr_batch *batch, int64_t *evals, int32_t *tile_q,
                        int32_t *chunk_q, int32_t *grid_ctas, int32_t *launches);
@@ -214,7 +217,8 @@ nr_status nr_plan_info(nr_ctx *ctx, const nr_batch *batch, int64_t *evals, int32
  * buckets; for i < min(*count, max_groups): nmax[i] the bucket's layer
  * capacity (1: exactly one layer; 0: any, forward), paired[i] 1 when the
  * two-evaluations-per-thread kernel runs it, tile_q[i] Q points per CTA
- * tile, grid[i] persistent CTAs, items[i] work items.  Arrays may be NULL. */
+ * tile, grid[i] consumers of the work queue (CTAs, or the 128-thread teams of
+ * the 3-and-more-layer gradients), items[i] work items.  Arrays may be NULL. */
 nr_status nr_plan_groups(nr_ctx *ctx, const nr_batch *batch, int32_t grad, int32_t max_groups, int32_t *count,
                          int32_t *nmax, int32_t *paired, int32_t *tile_q, int32_t *grid, int32_t *items);
 
