@@ -383,6 +383,19 @@ def test_common_quantum(order):
     assert_parity(wl, run_gpu(wl), run_oracle(wl))
 
 
+def test_gradient_on_a_waveguide_resonance():
+    """One quadrature node near a guided mode carries most of a gradient
+    component.  In a 64-bit evaluation of this stack a relative change of
+    6e-8 (one FP32 rounding) of the wavevectors inside the Fresnel factors
+    moves the scaled gradient by up to 1.1e-4, of r or the recursion's b by
+    7e-5 and 4e-5, of the phases by 8e-5: together 1.6e-4; 2e-4 with the
+    approximate special functions' share.  Wavevectors off by three roundings
+    exceed it."""
+    wl = W.make_workload("vi_step").subset([86])
+    gpu, ref = run_gpu(wl, modes=("grad",)), run_oracle(wl, modes=("grad",))
+    assert gpu["flags"] == 0 and grad_err(wl, gpu["g"], ref["g"]) < 2e-4
+
+
 def test_a_bad_q_point_leaves_the_others():
     """A non-positive or NaN Q point raises the flag and spoils its own model
     value only."""
