@@ -480,8 +480,7 @@ struct StackSmem {
     float4 med[NM + 2]; // medium j = 1..n+1: 4 pi (rho_j - rho_0) as (hi, lo), 4 pi iota_j, its square
     float4 itf[NM + 1]; // interface j = 0..n: 4 pi (rho_{j+1} - rho_j) + 4 pi i (iota_j - iota_{j+1}),
                         // s_j = -2 sigma_j^2, s_j log2(e)
-    float4 lay[NM + 2]; // layer j = 1..n: 2 d_j in table steps (x 128 / 2 pi) as (hi, lo), -2 d_j log2(e);
-                        // 4 pi (iota_{j-1} + iota_j) of the media above and in it (j = 1..n+1)
+    float4 lay[NM + 2]; // layer j = 1..n: 2 d_j in table steps (x 128 / 2 pi) as (hi, lo), -2 d_j log2(e), -
     float sig[NM + 1];  // sigma_j, j = 0..n
     float4 adj[NM + 1]; // interface j = 0..n: the adjoint's constants Re(s_j conj(N_j)) + 2 and - 2,
                         // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
@@ -513,9 +512,8 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
     const bool on = j <= n + 1, med = on && j >= 1, itf = j <= n, layer = med && itf;
     const double rho0 = p[n], rj = on ? p[n + j] : 0.0, ij = med ? p[2 * n + 1 + j] : 0.0;
     const double dj = layer ? p[j - 1] : 0.0, sig = itf ? p[3 * n + 3 + j] : 0.0;
-    const float aj = (float)(kFourPiD * ij); // 4 pi iota_j; its neighbours'
-    float aup = __shfl_up_sync(kFull, aj, 1), adn = __shfl_down_sync(kFull, aj, 1);
-    if (lane == 0 && j >= 2 && on) aup = (float)(kFourPiD * p[2 * n + j]);
+    const float aj = (float)(kFourPiD * ij); // 4 pi iota_j; its lower neighbour's
+    float adn = __shfl_down_sync(kFull, aj, 1);
     if (lane == 31 && itf) adn = (float)(kFourPiD * p[2 * n + 2 + j]);
     bool bad = !finite_bits(rj) || !finite_bits(ij) || !finite_bits(dj) || !finite_bits(sig);
     if (med) {
@@ -524,7 +522,7 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
     }
     if (on) {
         const float2 d2 = split_double(dj * kTwoStepsD);
-        sm.lay[j] = make_float4(d2.x, d2.y, (float)(-2.0 * kLog2ED * dj), j >= 1 ? aup + aj : 0.f);
+        sm.lay[j] = make_float4(d2.x, d2.y, (float)(-2.0 * kLog2ED * dj), 0.f);
     }
     if (itf) {
         const float dn = j < n ? 2.f * (float)p[j] : 0.f;

@@ -14,13 +14,12 @@
 // nothing is swapped between the halves, which would cost moves.
 //
 // The recursion runs in projective form (nr_pair.cuh), Nevot-Croce phases come
-// from a polynomial where the stack's roughnesses allow it, layer phases are
-// staged in table steps, and the Fresnel factor takes S^2 from the media's
-// known k^2.  Against the Moebius form with table phases, the later changes
-// below included: 16384 one-layer stacks x 400 Q x 21 nodes, gradient 1.464
-// -> 1.292 ms, log-likelihood 0.820 -> 0.749 ms; 12288 ten-layer stacks, model
-// curves 1.779 -> 1.426 ms; 10000 stacks of 1-20 layers, log-likelihood 1.623
-// -> 1.407 ms.
+// from a polynomial where the stack's roughnesses allow it, and layer phases
+// are staged in table steps.  Against the Moebius form with table phases, the
+// later changes below included: 16384 one-layer stacks x 400 Q x 21 nodes,
+// gradient 1.464 -> 1.292 ms, log-likelihood 0.820 -> 0.749 ms; 12288
+// ten-layer stacks, model curves 1.779 -> 1.426 ms; 10000 stacks of 1-20
+// layers, log-likelihood 1.623 -> 1.407 ms.
 //
 // The forward modes run the same code up to the smearing sum (model: write
 // scale S + bkg; log-likelihood: the residual terms) and no adjoint.
@@ -386,11 +385,11 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             auto fwd_step = [&](int j, auto TOP, auto BOT, auto TRIG) __attribute__((always_inline)) {
                 const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                 Kz2 kj;
-                if (top) kj = Kz2{k0h, bc(0.f), k0l, QUANT ? padd(p_hi, p_lo) : p_hi, bc(0.f)};
-                else kj = medium_kz2<TAB ? kRootFull : kRootPhase, QUANT>(p_hi, p_lo, sm.med[j]);
+                if (top) kj = Kz2{k0h, bc(0.f), k0l, bc(0.f)};
+                else kj = medium_kz2<kRootPhase, QUANT>(p_hi, p_lo, sm.med[j]);
                 const float4 Ij = sm.itf[j];
-                const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs)
-                                  : fresnel_g2<false, decltype(TRIG)::value>(kj, kbelow, Ij, sm.lay[j + 1].w, sh_cs);
+                const c2 Gj = top ? fresnel_g2<true, decltype(TRIG)::value>(kj, kbelow, Ij, sh_cs)
+                                  : fresnel_g2<false, decltype(TRIG)::value>(kj, kbelow, Ij, sh_cs);
                 const c2 rj = cscl2(Ij.x, Ij.y, Gj);
                 if (bot) {
                     B = rj;
@@ -511,7 +510,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                     const f2 mR = pneg(pmul(Rb2, R));
                     c2 Ab = c2{pmul(iA.re, mR), pneg(pmul(iA.im, mR))};
                     c2 kbar = czero();
-                    Kz2 kj = Kz2{k0h, bc(0.f), k0l, p_hi, bc(0.f)};
+                    Kz2 kj = Kz2{k0h, bc(0.f), k0l, bc(0.f)};
                     c2 Xb_up = czero(); // Xbar_{j-1} (edge sweeps)
                     const bool reach[2] = {lane_on[0] && qd[0].w < 0.f, lane_on[1] && qd[1].w < 0.f};
                     Kz2 kjm1 = kj;

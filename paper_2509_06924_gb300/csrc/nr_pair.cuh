@@ -92,25 +92,22 @@ __device__ __forceinline__ c2 cfmac2(c2 a, c2 b, c2 c)
     return c2{pfma(a.re, b.re, pfma(a.im, b.im, c.re)), pfma(a.re, b.im, pfma(pneg(a.im), b.re, c.im))};
 }
 
-// wavevector of both evaluations (value + low word of Re k, as Kz), its
-// square's real part u and 1 / |k|^2, by-products of the root
+// wavevector of both evaluations (value + low word of Re k, as Kz) and
+// 1 / |k|^2, a by-product of the root
 struct Kz2 {
-    f2 re, im, lo, u, y;
+    f2 re, im, lo, y;
 };
 __device__ __forceinline__ c2 kc2(const Kz2 &k) { return c2{k.re, k.im}; }
 
 // What is kept of a root's refinement.  kRootPlain: nothing (the backing, and
 // adjoint factors).  kRootPhase: the correction of Re k as a low word, which
-// only the phase takes.  kRootFull: Re k itself rounded from the exact root
-// too (two more additions).  Two approximate reciprocal roots leave t up to
-// three roundings off; (k_a + k_b)^2 let such an error of a shared k cancel
-// between two interfaces, S^2 from the known squares + 2 k_a k_b does not.
-// Worst scaled gradient error of 1632 twelve-layer stacks 3.3e-4 with
-// kRootPhase (on a waveguide resonance whose gradient moves by 5e-5 to 8e-5
-// with its inputs' roundings), 1.1e-4 with kRootFull, the 99.9 % quantile
-// 3.2e-5 and 1.7e-5, for 0.5 % of the time.  The log-likelihood sums every
-// point and needs no more than kRootPhase (its errors are no larger with it,
-// and its kernel is 2.5 % faster).
+// only the phase takes (t, two approximate reciprocal roots, is up to three
+// roundings off; the same t in both interfaces' k_a + k_b leaves most of it to
+// cancel).  kRootFull: Re k itself rounded from the exact root too (two more
+// additions, 0.5 % of the time): the deep gradients, where a waveguide
+// resonance carries whatever does not cancel (1632 twelve-layer stacks, 99.9 %
+// quantile of the scaled gradient's error 2.4e-5 with kRootPhase, 2.3e-5 with
+// kRootFull; the worst stack 1.9e-4 and 1.3e-4).
 enum : int { kRootPlain = 0, kRootPhase = 1, kRootFull = 2 };
 
 // principal sqrt of u + i a (u = uh + ul, a >= 0 the stack's 4 pi iota,
@@ -119,7 +116,6 @@ template <int REFINE>
 __device__ __forceinline__ Kz2 kz_sqrt2(f2 uh, f2 ul, float a, float a2)
 {
     Kz2 k;
-    k.u = uh;
     const f2 au = pabs(uh);
     const f2 m2 = pfma(uh, uh, bc(a2));
     k.y = prsqrt(pmax(m2, bc(1e-37f)));
@@ -199,17 +195,22 @@ __device__ __forceinline__ c2 layer_phase2(const Kz2 &k, float4 L, const float *
 }
 
 // G = exp(s k_a k_b) / S^2, S = k_a + k_b: the Nevot-Croce Fresnel
-// coefficient without its numerator, r = N G.  S^2 = k_a^2 + k_b^2 + 2 k_a k_b
-// takes the squares as they are known (u_a + u_b + i aa, aa the sum of both
-// media's 4 pi iota), and G = w (cos + i sin) conj(S^2) with w = exp(s Re) /
-// |S^2|^2.  REAL_A: k_a is real (the fronting medium).  A vanishing S
-// (k_a = k_b = 0) gives a finite G whose numerator is 0.
+// coefficient without its numerator, r = N G.  G = w (cos + i sin) conj(S^2)
+// with w = exp(s Re) / |S^2|^2.  S is the sum itself: an error of k_j then
+// enters the interfaces above and below it alike and mostly cancels, which
+// S^2 = k_a^2 + k_b^2 + 2 k_a k_b from the known squares does not allow.  That
+// form saves three operations (log-likelihoods 0-2 % faster) and left thick
+// films a larger error of the gradient call's log-likelihood (99 % quantile of
+// 1500: 6.3e-7 against 5.0e-7) and of the gradient (median 4.1e-7, 3.6e-7).
+// REAL_A: k_a is real (the fronting medium).  A vanishing S (k_a = k_b = 0)
+// gives a finite G whose numerator is 0.
 template <bool REAL_A, int TRIG>
-__device__ __forceinline__ c2 fresnel_g2(const Kz2 &ka, const Kz2 &kb, float4 I, float aa, const float *tab)
+__device__ __forceinline__ c2 fresnel_g2(const Kz2 &ka, const Kz2 &kb, float4 I, const float *tab)
 {
     const c2 kk = REAL_A ? c2{pmul(ka.re, kb.re), pmul(ka.re, kb.im)} : cmul2(kc2(ka), kc2(kb));
-    const f2 A = pfma(bc(2.f), kk.re, padd(ka.u, kb.u)); // Re S^2
-    const f2 B = pfma(bc(2.f), kk.im, bc(aa));           // Im S^2
+    const f2 Sx = padd(ka.re, kb.re), Sy = REAL_A ? kb.im : padd(ka.im, kb.im);
+    const f2 A = pfma(Sx, Sx, pneg(pmul(Sy, Sy))); // Re S^2
+    const f2 B = pmul(padd(Sx, Sx), Sy);           // Im S^2
     const f2 inv = prcp(pmax(pfma(A, A, pmul(B, B)), bc(1e-36f)));
     const f2 w = pmul(pex2(pmul(bc(I.w), kk.re)), inv);
     const f2 ph = pmul(bc(I.z), kk.im);

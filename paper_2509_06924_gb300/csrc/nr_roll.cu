@@ -373,7 +373,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 {
                     const Kz2 kj = medium_kz2<kRootFull, true>(p_hi, p_lo, sm.med[n]);
                     const float4 I = sm.itf[n];
-                    const c2 G = fresnel_g2<false, T>(kj, kb, I, sm.lay[n + 1].w, sh_cs);
+                    const c2 G = fresnel_g2<false, T>(kj, kb, I, sh_cs);
                     B = cscl2(I.x, I.y, G);
                     ts.b[NM * kTeam + tid] = make_float4(G.re.x, G.re.y, G.im.x, G.im.y);
                     kb = kj;
@@ -381,11 +381,11 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 auto step = [&](int j, auto TOP) __attribute__((always_inline)) {
                     constexpr bool top = decltype(TOP)::value;
                     Kz2 kj;
-                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, padd(p_hi, p_lo), bc(0.f)};
+                    if constexpr (top) kj = Kz2{k0h, bc(0.f), k0l, bc(0.f)};
                     else kj = medium_kz2<kRootFull, true>(p_hi, p_lo, sm.med[j]);
                     const float4 I = sm.itf[j];
                     const float4 L = sm.lay[j + 1];
-                    const c2 G = fresnel_g2<top, T>(kj, kb, I, L.w, sh_cs);
+                    const c2 G = fresnel_g2<top, T>(kj, kb, I, sh_cs);
                     const c2 E = layer_phase2<true>(kb, L, sh_cs);
                     tmem_store(tm + j * kSlotCols, G, E);
                     const c2 r = cscl2(I.x, I.y, G);
