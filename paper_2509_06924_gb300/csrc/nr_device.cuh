@@ -27,15 +27,14 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // |k_j|^2 < kEdgeFrac k_0^2 selects the interior-edge treatment of the adjoint.
 // Outside the band the plain adjoint loses about k_0^2 / |k_j|^2 roundings of an
-// evaluation's own term, on an ever smaller share of the evaluations.  Bands
-// of 0.04, 0.02, 0.01 and 0.005 give the same errors against the oracle on
-// 200 ten-layer chains (median 3.5e-7, 99 % within 2.7e-6), 60 twelve-layer
-// ones (8.1e-7, 7.2e-6), 1500 thick films (2.2e-7, 2.1e-6), 1024 thin films and
-// 400 uneven stacks; a band of 0.01 queues a quarter of 0.04's entries:
-// twelve-layer gradients 26.2 -> 25.4 ms (49152 stacks), ten-layer 3.51 ->
-// 3.38 ms, 21-64 layers 1.78 -> 1.67 ms.
+// evaluation's own term.  Whole smeared curves average that away (200 to 1500
+// stacks of five kinds: the same errors with bands from 0.005 to 0.04), an
+// unsmeared point does not: 600 one- to ten-layer stacks with one point each,
+// k_j^2 at 1 to 4 % of k_0^2, scaled gradient errors of the worst tenth from
+// 4e-5 with a band of 0.04 and from 8e-4 with 0.01.  The wider band costs
+// twelve-layer gradients 3 %, ten-layer ones 4 %, 21 to 64 layers 6 %.
 #ifndef NR_EDGE_FRAC
-#define NR_EDGE_FRAC 0.01f
+#define NR_EDGE_FRAC 0.04f
 #endif
 constexpr float kEdgeFrac = NR_EDGE_FRAC;
 
