@@ -86,6 +86,11 @@ __device__ __forceinline__ c2 cmulc2(c2 a, c2 b)
 {
     return c2{pfma(a.re, b.re, pmul(a.im, b.im)), pfma(a.re, b.im, pneg(pmul(a.im, b.re)))};
 }
+// 1 - a^2
+__device__ __forceinline__ c2 one_minus_sq2(c2 a)
+{
+    return c2{pfma(pneg(a.re), a.re, pfma(a.im, a.im, bc(1.f))), pmul(bc(-2.f), pmul(a.re, a.im))};
+}
 // conj(a) * b + c
 __device__ __forceinline__ c2 cfmac2(c2 a, c2 b, c2 c)
 {

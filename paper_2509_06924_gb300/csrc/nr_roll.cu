@@ -306,17 +306,16 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     v.y = 0.5f * fsc * __ldg(dqp + qa);
                     v.z = __ldg(rop + qa);
                     v.w = rcp_approx(__ldg(rep + qa));
-                    // may a node of this Q point reach an interior-edge band?
-                    // (negative 1/err: yes)
+                    // may a node of this Q point lie below an interior edge or
+                    // reach its band?  (negative 1/err: yes)
                     const float a = fabsf(v.y) * g_max;
                     const float lo = fmaxf(v.x - a, 0.f), hi = v.x + a;
                     p_bits = max(p_bits, quantum_bits(hi * hi));
                     const float k2lo = lo * lo * (1.f - 1.5f * kEdgeFrac);
-                    const float k2hi = hi * hi * (1.f + 1.5f * kEdgeFrac);
                     bool e = false;
                     for (int j = 1; j <= n; ++j) {
                         const float c = sm.med[j].x + sm.med[j].y;
-                        e |= c > 0.f && c < k2hi && c > k2lo;
+                        e |= c > 0.f && c > k2lo;
                     }
                     if (e && v.w > 0.f) v.w = -v.w;
                 }
@@ -442,6 +441,16 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             // Xbar_0 = 2 Rbar X_0: Bbar_0 = Xbar_0 / conj(A_0), Abar_0 =
             // -conj(X_0) Bbar_0; every step applies the conjugate transpose of
             // the forward one.  A_{j+1} = A_j - r_j b_j runs the forward's A back.
+            // Abar and Bbar cancel where the reflectivity is near 1 (their common
+            // scale is free, and roundings along it are amplified); there the sweep
+            // carries Z_j = Bbar_j / conj(A_j) alone:
+            //   rbar_j = conj(A_{j+1}^2 - b_j^2) Z_j,  bbar_j = conj(A_{j+1}) t_j,
+            //   Z_{j+1} = conj(E_{j+1}) t_j,  t_j = conj(1 - r_j^2) Z_j,
+            // eight operations a layer more, as accurate as the Moebius form.
+            // Layers' gradients of 600 unsmeared points below an edge, 90 % within
+            // 9.8e-5 (4 layers), 2.9e-4 (10), 1.3e-3 (40) with Abar and Bbar,
+            // 2.9e-5, 4.4e-5, 5.6e-5 with Z.  On the tiles that need it it costs the
+            // ten- and twelve-layer gradients 1 %.
             const f2 Rb2 = padd(Rb, Rb);
             c2 Bb = cmulc2(iA, X0);
             Bb = c2{pmul(Bb.re, Rb2), pmul(Bb.im, Rb2)};
@@ -455,6 +464,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
             const f2 wres = RES ? pmul(dQh, g_hi) : bc(0.f);
             f2 res_sum = bc(0.f), res_k0 = bc(0.f);
+            // EDG: Bb holds Z, Ab is not used
             auto adj_step = [&](int j, auto TOP, auto BOT, auto EDG) __attribute__((always_inline)) {
                 constexpr bool top = decltype(TOP)::value, bot = decltype(BOT)::value, edg = decltype(EDG)::value;
                 // G_j, E_{j+1}: the load runs while k_{j+1} is formed (never across a
@@ -468,7 +478,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 c2 G, b = czero(), kbar1 = czero(), rb = Bb, Xb_in = czero();
                 f2 accD = bc(0.f);
                 float2 Z[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                if constexpr (edg) Xb_in = cmulc2(A, Bb);
+                if constexpr (edg) Xb_in = cmulc2(A, cmulc2(A, Bb));
                 if constexpr (bot) {
                     G = c2{make_float2(bv.x, bv.y), make_float2(bv.z, bv.w)};
                 } else {
@@ -478,12 +488,21 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     b = c2{make_float2(bv.x, bv.y), make_float2(bv.z, bv.w)};
                     const c2 r = cscl2(I.x, I.y, G);
                     A = cfnma2(r, b, A);                  // A_{j+1}
-                    rb = cfmac2(b, Ab, cmulc2(A, Bb));
                     // adjoint of b = E B: with U = conj(b) bbar the thickness sum
                     // takes Im(conj(k) U) and kbar_{j+1} gets -2 i d U
-                    const c2 bb = cfmac2(r, Ab, Bb);
-                    Ab = cfmac2(r, Bb, Ab);
-                    Bb = cmulc2(E, bb);
+                    c2 bb;
+                    if constexpr (edg) {
+                        const c2 s = cadd2(A, b), d = c2{psub(A.re, b.re), psub(A.im, b.im)};
+                        rb = cmulc2(cmul2(s, d), Bb);
+                        const c2 t = cmulc2(one_minus_sq2(r), Bb);
+                        bb = cmulc2(A, t);
+                        Bb = cmulc2(E, t);
+                    } else {
+                        rb = cfmac2(b, Ab, cmulc2(A, Bb));
+                        bb = cfmac2(r, Ab, Bb);
+                        Ab = cfmac2(r, Bb, Ab);
+                        Bb = cmulc2(E, bb);
+                    }
                     const c2 U = cmulc2(b, bb);
                     accD = pfma(kj1.re, U.im, pneg(pmul(kj1.im, U.re)));
                     kbar1 = c2{pmul(bc(C.w), U.im), pneg(pmul(bc(C.w), U.re))};
@@ -552,13 +571,14 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 }
             };
             auto sweep = [&](auto EDG) __attribute__((always_inline)) {
+                if constexpr (decltype(EDG)::value) Bb = cmulc2(iA, Bb); // Z_0
                 adj_step(0, std::true_type{}, std::false_type{}, EDG);
 #pragma unroll 1
                 for (int j = 1; j <= n - 1; ++j) adj_step(j, std::false_type{}, std::false_type{}, EDG);
                 adj_step(n, std::false_type{}, std::true_type{}, EDG);
             };
-            // the staged sign of 1/err marks Q points whose nodes may reach an
-            // interior-edge band (warp-uniform choice)
+            // the staged sign of 1/err marks Q points whose nodes may lie below an
+            // interior edge or in its band (warp-uniform choice)
             if (__any_sync(kFull, reach[0] || reach[1])) sweep(std::true_type{});
             else sweep(std::false_type{});
             if constexpr (RES) gres_acc = pfma(wres, pfma(k0h, res_sum, res_k0), gres_acc);

@@ -443,6 +443,19 @@ def test_unsmeared_points_near_an_interior_edge(n):
     assert np.quantile(layer_grad_err(wl, n), 0.9) <= TOL_G
 
 
+# The same for deeper stacks, and for points below an edge (k_j^2 down to
+# -k_0^2): near total reflection the adjoint of a recursion without divisions
+# cancels from layer to layer unless it carries the one combination that does
+# not.  Bounds: nine of ten stacks within the errors of a kernel that
+# differentiates the division itself (`q90`), with 30 % for the spread of that
+# quantile over 600 stacks.
+@pytest.mark.parametrize("n,lo,hi,q90", [(10, 0.0102, 0.0398, 5.62e-5), (20, 0.0102, 0.0398, 8.15e-5),
+                                         (2, -1.0, -0.05, 3.40e-5), (4, -1.0, -0.05, 3.83e-5),
+                                         (10, -1.0, -0.05, 5.09e-5), (40, -1.0, -0.05, 6.66e-5)])
+def test_unsmeared_points_in_total_reflection(n, lo, hi, q90):
+    assert np.quantile(layer_grad_err(edge_points(n, lo, hi), n), 0.9) <= 1.3 * q90
+
+
 def test_a_bad_q_point_leaves_the_others():
     """A non-positive or NaN Q point raises the flag and spoils its own model
     value only."""
