@@ -474,6 +474,19 @@ __device__ __forceinline__ int queue_count(int cnt)
 
 // Per-stack parameters staged in shared memory, one 16-byte entry per
 // medium, interface and layer (a sweep step reads each with one load).
+// What a stack's roughnesses ask of the paired kernels.
+// kNcBig: some interface's Nevot-Croce phase may exceed kNcSmall (table).
+// kNcGrows (with kNcBig): the projective recursion may overflow.  Between two
+// evanescent media the factor exp(-2 sigma^2 k_a k_b) grows, |r_j| <= g_j =
+// exp(2 sigma^2 Im k_a Im k_b) with Im k^2 <= max(c, 0) + a / 2, and max(|A|,
+// |B|) by 1 + |r_j| <= 2 g_j a layer.  A warp stages 32 interfaces; where the
+// sum of its log2 g_j passes kNcGrowth the kernels divide by A_j at every
+// layer, and elsewhere |A_0| <= 2^(n + 5 ceil((n + 2) / 32)), 2^25 up to 20
+// layers.  Ordinary stacks stay far below (20 layers, sigma 20 A, SLDs of
+// 6e-6 throughout: 1.7).
+enum : int { kNcBig = 1, kNcGrows = 2 };
+constexpr float kNcGrowth = 5.f;
+
 template <int NM>
 struct StackSmem {
     float4 med[NM + 2]; // medium j = 1..n+1: 4 pi (rho_j - rho_0) as (hi, lo), 4 pi iota_j, its square
@@ -485,8 +498,8 @@ struct StackSmem {
                         // Im(s_j conj(N_j)) (N_j the interface's complex SLD step); 2 d_{j+1}
     float scale, bkg;
     int p_max;          // bits of the largest k_0^2 or |c_j| of the item so far (split_media)
-    int nc_big[2];      // 1: some interface's Nevot-Croce phase may exceed kNcSmall (cleared by the item's
-                        // owner; two, so that an item can clear the next one's)
+    int nc_big[2];      // kNcBig, kNcGrows (cleared by the item's owner; two, so that an item can clear
+                        // the next one's)
 };
 
 __device__ __forceinline__ float2 split_double(double v)
@@ -515,21 +528,27 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
     float adn = __shfl_down_sync(kFull, aj, 1);
     if (lane == 31 && itf) adn = (float)(kFourPiD * p[2 * n + 2 + j]);
     bool bad = !finite_bits(rj) || !finite_bits(ij) || !finite_bits(dj) || !finite_bits(sig);
+    float up = 0.f; // the largest Im k_j^2, and its lower neighbour's
     if (med) {
         const float2 c = split_double(kFourPiD * (rj - rho0));
         sm.med[j] = make_float4(c.x, c.y, aj, aj * aj);
+        up = fmaxf(c.x, 0.f) + 0.5f * fabsf(aj);
     }
+    float dn = __shfl_down_sync(kFull, up, 1);
+    if (lane == 31 && itf) dn = fmaxf((float)(kFourPiD * (p[n + j + 1] - rho0)), 0.f) + 0.5f * fabsf(adn);
+    bool big = false;
+    int grows = 0; // log2 of the interface's growth in 1/64
     if (on) {
         const float2 d2 = split_double(dj * kTwoStepsD);
         sm.lay[j] = make_float4(d2.x, d2.y, (float)(-2.0 * kLog2ED * dj), 0.f);
     }
     if (itf) {
-        const float dn = j < n ? 2.f * (float)p[j] : 0.f;
+        const float d2n = j < n ? 2.f * (float)p[j] : 0.f;
         const float Nr = (float)(kFourPiD * (p[n + j + 1] - rj)), Ni = aj - adn;
         const double sig2 = sig * sig;
         const float s = -2.f * (float)sig2;
         sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig2));
-        sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, dn);
+        sm.adj[j] = make_float4(fmaf(s, Nr, 2.f), fmaf(s, Nr, -2.f), -s * Ni, d2n);
         sm.sig[j] = (float)sig;
         // |s Im(k_j k_{j+1})| <= -s (D / 2 + sqrt(5 m a) + a) with
         // D = |Re N|, a the larger 4 pi iota of the two media, m = max(D, a):
@@ -538,8 +557,12 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
         // + 2 a a'; for |u| > 4 m of one sign it is below (0.6 (a + a'))^2 x 2
         const float D = fabsf(Nr), a = fmaxf(fabsf(aj), fabsf(adn));
         const float bound = -s * (0.5f * D + sqrtf(5.f * fmaxf(D, a) * a) + 1.2f * a);
-        if (!(bound <= kNcSmall)) *nc_big = 1; // every writer stores the same value
+        big = !(bound <= kNcSmall);
+        grows = (int)fminf((float)(2.0 * kLog2ED * 64.0) * (float)sig2 * sqrtf(up) * sqrtf(dn), 1e6f);
     }
+    grows = __reduce_add_sync(kFull, grows) > (int)(64.f * kNcGrowth) ? kNcGrows | kNcBig : 0;
+    grows |= __any_sync(kFull, big) ? kNcBig : 0;
+    if (lane == 0 && grows) atomicOr(nc_big, grows);
     if (j == 0) {
         const double scale = p[4 * n + 4], bkg = p[4 * n + 5];
         sm.scale = (float)scale;

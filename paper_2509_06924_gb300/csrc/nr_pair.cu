@@ -382,6 +382,7 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             c2 rst[NK], Gst[NK], Est[NK], bst[NK], Ast[NK];
             c2 A = c2{bc(1.f), bc(0.f)}, B = czero();
             Kz2 kbelow = medium_kz2<kRootPlain, QUANT>(p_hi, p_lo, sm.med[n + 1]);
+            bool renorm = false; // divide by A at every interface
             auto fwd_step = [&](int j, auto TOP, auto BOT, auto TRIG) __attribute__((always_inline)) {
                 const bool top = pos_flag(TOP, j == 0), bot = pos_flag(BOT, j == n);
                 Kz2 kj;
@@ -405,6 +406,12 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                         const c2 An = A;
                         A = cfma2(rj, b, An);
                         B = cfma2(rj, An, b);
+                        if constexpr (PT::RFWD && decltype(TRIG)::value == kTrigTable) {
+                            if (renorm) {
+                                B = cmul2(B, cinv2(A));
+                                A = c2{bc(1.f), bc(0.f)};
+                            }
+                        }
                     }
                     if constexpr (GRAD) {
                         Est[j + 1] = Ej;
@@ -431,15 +438,21 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
                         if (j <= n) fwd_step(j, Pos<kRt>{}, Pos<kRt>{}, TRIG);
                 }
             };
-            if constexpr (!TAB) forward(Pos<kTrigMufu>{});
-            else if (sm.nc_big[par]) forward(Pos<kTrigTable>{});
-            else forward(Pos<kTrigSmall>{});
-            // X_0 = B_0 / A_0 and R = |X_0|^2; |A_0| <= 2^n needs scaling only in
-            // the deepest bucket
+            const int nc = sm.nc_big[par];
+            renorm = nc & kNcGrows;
+            if constexpr (!TAB) {
+                if (PT::RFWD && renorm) forward(Pos<kTrigTable>{});
+                else forward(Pos<kTrigMufu>{});
+            } else {
+                if (nc) forward(Pos<kTrigTable>{});
+                else forward(Pos<kTrigSmall>{});
+            }
+            // X_0 = B_0 / A_0 and R = |X_0|^2; |A_0| (kNcGrows) needs scaling in
+            // the deepest bucket, and in the gradient of two layers that may grow
             c2 iA = czero(), X0 = czero();
             f2 R;
             if constexpr (GRAD || NMAX > 20) {
-                if constexpr (NMAX > 20) {
+                if (NMAX > 20 || (NMAX == 2 && renorm)) {
                     iA = cinv2(A);
                 } else {
                     const f2 iv = prcp(pfma(A.re, A.re, pmul(A.im, A.im)));

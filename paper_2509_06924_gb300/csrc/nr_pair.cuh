@@ -233,6 +233,7 @@ __device__ __forceinline__ c2 fresnel_g2(const Kz2 &ka, const Kz2 &kb, float4 I,
 // Against X_j = (r_j + Y) / (1 + r_j Y), Y = E_{j+1} X_{j+1}, it needs no
 // division per interface (12 operations for 19 and two reciprocals) and its
 // chain from one interface to the next is four dependent operations long.
+// Stacks whose A would overflow (kNcGrows) divide by it after every interface.
 // a b + c
 __device__ __forceinline__ c2 cfma2(c2 a, c2 b, c2 c)
 {

@@ -334,7 +334,8 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
         team_sync(team);
 
         const float scale = sm.scale, bkg = sm.bkg;
-        const bool nc_big = sm.nc_big[0] != 0;
+        const int nc = sm.nc_big[0];
+        const bool renorm = nc & kNcGrows; // divide by A at every interface
         const f2 wks = pmul(wk, bc(scale));
         int buf = 0;
         // t0: the tile's first Q point within the staged super-tile.  Slots past
@@ -392,13 +393,19 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     ts.b[j * kTeam + tid] = make_float4(b.re.x, b.re.y, b.im.x, b.im.y);
                     B = cfma2(r, A, b);
                     A = cfma2(r, b, A);
+                    if constexpr (T == kTrigTable) {
+                        if (renorm) {
+                            B = cmul2(B, cinv2(A));
+                            A = c2{bc(1.f), bc(0.f)};
+                        }
+                    }
                     kb = kj;
                 };
 #pragma unroll 1
                 for (int j = n - 1; j >= 1; --j) step(j, std::false_type{});
                 step(0, std::true_type{});
             };
-            if (nc_big) forward(Pos<kTrigTable>{});
+            if (nc) forward(Pos<kTrigTable>{});
             else forward(Pos<kTrigSmall>{});
             const c2 iA = cinv2(A); // 1 / A_0
             const c2 X0 = cmul2(B, iA);
@@ -464,8 +471,9 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
             const f2 edge_u = pmul(bc(kEdgeFrac), pmul(k0h, k0h));
             const f2 wres = RES ? pmul(dQh, g_hi) : bc(0.f);
             f2 res_sum = bc(0.f), res_k0 = bc(0.f);
-            // EDG: Bb holds Z, Ab is not used
-            auto adj_step = [&](int j, auto TOP, auto BOT, auto EDG) __attribute__((always_inline)) {
+            // EDG: Bb holds Z, Ab is not used; REN (stacks divided by A at every
+            // interface): A_j = 1, Bb holds Xbar_j between the steps
+            auto adj_step = [&](int j, auto TOP, auto BOT, auto EDG, auto REN) __attribute__((always_inline)) {
                 constexpr bool top = decltype(TOP)::value, bot = decltype(BOT)::value, edg = decltype(EDG)::value;
                 // G_j, E_{j+1}: the load runs while k_{j+1} is formed (never across a
                 // loop iteration: its registers may not be copied before the wait)
@@ -478,7 +486,6 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                 c2 G, b = czero(), kbar1 = czero(), rb = Bb, Xb_in = czero();
                 f2 accD = bc(0.f);
                 float2 Z[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                if constexpr (edg) Xb_in = cmulc2(A, cmulc2(A, Bb));
                 if constexpr (bot) {
                     G = c2{make_float2(bv.x, bv.y), make_float2(bv.z, bv.w)};
                 } else {
@@ -487,7 +494,15 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     const c2 E = c2{sl.c, sl.d};
                     b = c2{make_float2(bv.x, bv.y), make_float2(bv.z, bv.w)};
                     const c2 r = cscl2(I.x, I.y, G);
-                    A = cfnma2(r, b, A);                  // A_{j+1}
+                    if constexpr (decltype(REN)::value) {
+                        const c2 rb1 = cmul2(r, b), iD = cinv2(c2{padd(bc(1.f), rb1.re), rb1.im});
+                        Xb_in = Bb;
+                        Bb = cmulc2(iD, cmulc2(iD, Bb));
+                        A = c2{bc(1.f), bc(0.f)};
+                    } else {
+                        if constexpr (edg) Xb_in = cmulc2(A, cmulc2(A, Bb));
+                        A = cfnma2(r, b, A); // A_{j+1}
+                    }
                     // adjoint of b = E B: with U = conj(b) bbar the thickness sum
                     // takes Im(conj(k) U) and kbar_{j+1} gets -2 i d U
                     c2 bb;
@@ -570,17 +585,18 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
                     if constexpr (RES) res_sum = padd(res_sum, ur);
                 }
             };
-            auto sweep = [&](auto EDG) __attribute__((always_inline)) {
-                if constexpr (decltype(EDG)::value) Bb = cmulc2(iA, Bb); // Z_0
-                adj_step(0, std::true_type{}, std::false_type{}, EDG);
+            auto sweep = [&](auto EDG, auto REN) __attribute__((always_inline)) {
+                if constexpr (decltype(EDG)::value) Bb = cmulc2(iA, Bb); // Z_0 (Xbar_0 where A_0 = 1)
+                adj_step(0, std::true_type{}, std::false_type{}, EDG, REN);
 #pragma unroll 1
-                for (int j = 1; j <= n - 1; ++j) adj_step(j, std::false_type{}, std::false_type{}, EDG);
-                adj_step(n, std::false_type{}, std::true_type{}, EDG);
+                for (int j = 1; j <= n - 1; ++j) adj_step(j, std::false_type{}, std::false_type{}, EDG, REN);
+                adj_step(n, std::false_type{}, std::true_type{}, EDG, REN);
             };
             // the staged sign of 1/err marks Q points whose nodes may lie below an
             // interior edge or in its band (warp-uniform choice)
-            if (__any_sync(kFull, reach[0] || reach[1])) sweep(std::true_type{});
-            else sweep(std::false_type{});
+            if (renorm) sweep(std::true_type{}, std::true_type{});
+            else if (__any_sync(kFull, reach[0] || reach[1])) sweep(std::true_type{}, std::false_type{});
+            else sweep(std::false_type{}, std::false_type{});
             if constexpr (RES) gres_acc = pfma(wres, pfma(k0h, res_sum, res_k0), gres_acc);
         }
         }

@@ -456,6 +456,37 @@ def test_unsmeared_points_in_total_reflection(n, lo, hi, q90):
     assert np.quantile(layer_grad_err(edge_points(n, lo, hi), n), 0.9) <= 1.3 * q90
 
 
+# Between two evanescent media the Nevot-Croce factor exp(-2 sigma^2 k_a k_b)
+# grows; products of it over the layers must not overflow as long as each
+# reflection stays finite.  Roughnesses from where the recursion is first
+# divided at every layer to where the products of 64 layers pass 1e90; thin and
+# thick layers, an absorbing stack.  Every output is finite, and the median
+# stack meets the module's bounds (guided modes behind such interfaces are
+# ill-conditioned beyond what input perturbations show: factors of e^20 carry
+# the roundings of their exponents).
+@pytest.mark.parametrize("n", [2, 3, 10, 20, 32, 64])
+def test_very_rough_evanescent_layers(n):
+    rng = np.random.default_rng(70 + n)
+    q = W.log_grid(40, 0.004, 0.02)
+    datasets, stacks = [], []
+    for sigma in (60.0, 120.0, 180.0, 220.0, 260.0, 320.0):
+        for d, iota in ((100.0, 0.0), (300.0, 0.0), (40.0, 1e-8)):
+            rho = np.where(np.arange(n) % 2, 6.3e-6, 3.5e-6) * rng.uniform(0.97, 1.03, n)
+            p = W.pack(np.full(n, d), np.concatenate([[0.0], rho, [6.3e-6]]), np.full(n + 1, iota),
+                       sigma * rng.uniform(0.95, 1.05, n + 1), 1.0, 1e-7)
+            stacks.append((n, p, len(datasets)))
+            datasets.append((q, 0.03 * q.astype(np.float64)))
+    wl = custom_workload(stacks, datasets)
+    gpu = run_gpu(wl)
+    assert gpu["flags"] == 0 and all(np.all(np.isfinite(gpu[k])) for k in ("m", "ll", "ll_g", "g"))
+    err = stack_errors(wl, gpu, run_oracle(wl))
+    for kind, tol in (("model", TOL_M), ("loglik", TOL_LL), ("loglik_g", TOL_LL), ("grad", TOL_G)):
+        assert np.median(err[kind]) <= tol
+    ctx = nr.Context(n_quad=wl.n_quad)
+    assert all(torch.isfinite(t).all() for t in ctx.loglik_grad_res(nr.Batch.from_workload(wl)))
+    ctx.close()
+
+
 def test_a_bad_q_point_leaves_the_others():
     """A non-positive or NaN Q point raises the flag and spoils its own model
     value only."""
