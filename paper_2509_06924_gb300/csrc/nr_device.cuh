@@ -524,14 +524,15 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
     const bool on = j <= n + 1, med = on && j >= 1, itf = j <= n, layer = med && itf;
     const double rho0 = p[n], rj = on ? p[n + j] : 0.0, ij = med ? p[2 * n + 1 + j] : 0.0;
     const double dj = layer ? p[j - 1] : 0.0, sig = itf ? p[3 * n + 3 + j] : 0.0;
-    const float aj = (float)(kFourPiD * ij); // 4 pi iota_j; its lower neighbour's
+    const double aj64 = kFourPiD * ij;
+    const float aj = (float)aj64; // 4 pi iota_j; its lower neighbour's
     float adn = __shfl_down_sync(kFull, aj, 1);
     if (lane == 31 && itf) adn = (float)(kFourPiD * p[2 * n + 2 + j]);
     bool bad = !finite_bits(rj) || !finite_bits(ij) || !finite_bits(dj) || !finite_bits(sig);
     float up = 0.f; // the largest Im k_j^2, and its lower neighbour's
     if (med) {
         const float2 c = split_double(kFourPiD * (rj - rho0));
-        sm.med[j] = make_float4(c.x, c.y, aj, aj * aj);
+        sm.med[j] = make_float4(c.x, c.y, aj, (float)(aj64 * aj64));
         up = fmaxf(c.x, 0.f) + 0.5f * fabsf(aj);
     }
     float dn = __shfl_down_sync(kFull, up, 1);
@@ -544,7 +545,8 @@ __device__ void stage_stack(StackSmem<NM> &sm, int *nc_big, const double *p, int
     }
     if (itf) {
         const float d2n = j < n ? 2.f * (float)p[j] : 0.f;
-        const float Nr = (float)(kFourPiD * (p[n + j + 1] - rj)), Ni = aj - adn;
+        // (differences in FP64: nearly equal media cancel)
+        const float Nr = (float)(kFourPiD * (p[n + j + 1] - rj)), Ni = (float)(kFourPiD * (ij - p[2 * n + 2 + j]));
         const double sig2 = sig * sig;
         const float s = -2.f * (float)sig2;
         sm.itf[j] = make_float4(Nr, Ni, s, (float)(-2.0 * kLog2ED * sig2));

@@ -487,6 +487,23 @@ def test_very_rough_evanescent_layers(n):
     ctx.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 4])
+def test_absorption_steps_between_nearly_equal_media(n):
+    """Equal SLDs and absorptions that differ by 1 part in 10^4, only in the last
+    interface, behind a surface too rough to reflect: what is measured is that
+    difference, which FP32 absorptions do not hold to better than 4e-4.  The
+    parameters are FP64: the module's bounds, without its allowance for FP32
+    roundings of the inputs."""
+    rho, iota = np.zeros(n + 2), np.full(n + 1, 1e-6)
+    iota[-1] *= 1.0001
+    sigma = np.concatenate([[70.0], np.full(n - 1, 5.0), [3.0]])
+    q = W.log_grid(60, 0.08, 0.12)
+    wl = custom_workload([(n, W.pack(np.full(n, 40.0), rho, iota, sigma, 1.0, 0.0), 0)],
+                         [(q, 0.02 * q.astype(np.float64))])
+    err = stack_errors(wl, run_gpu(wl), run_oracle(wl))
+    assert err["model"] <= TOL_M and max(err["loglik"], err["loglik_g"]) <= TOL_LL and err["grad"] <= TOL_G
+
+
 def test_a_bad_q_point_leaves_the_others():
     """A non-positive or NaN Q point raises the flag and spoils its own model
     value only."""
