@@ -819,6 +819,36 @@ def test_sld_profile_runs(nz, order):
     ctx.close()
 
 
+def test_sld_profile_sharp_steps_on_grid_depths():
+    """Sharp steps whose depths, added up in FP64 from thicknesses in tenths, lie
+    on float grid points take the deeper medium's value there, in stacks of more
+    interfaces than a warp has lanes too."""
+    rng = np.random.default_rng(3)
+    stacks, zs = [], set()
+    for n in np.repeat([2, 5, 8, 40], 60):
+        st = rand_stack(rng, int(n))
+        L = W.layout(int(n))
+        st[L["d"]] = np.round(rng.uniform(5, 300, n), 1)
+        st[L["sigma"]] = 0.0
+        stacks.append((int(n), st, 0))
+        depth = 0.0
+        for d in st[L["d"]]:
+            depth += d
+            if float(np.float32(depth)) == depth:
+                zs.add(depth)
+    z = np.array(sorted(zs), np.float32)
+    q = W.log_grid(10, 0.01, 0.2)
+    wl = custom_workload(stacks, [(q, 0.05 * q.astype(np.float64))])
+    ctx = nr.Context(n_quad=wl.n_quad)
+    rho = ctx.sld_profile(nr.Batch.from_workload(wl), torch.as_tensor(z, device="cuda"))[0]
+    ctx.close()
+    for (n, st, _), got in zip(stacks, rho):
+        depth = np.cumsum(st[W.layout(n)["d"]])  # sequential, as the library adds
+        want = st[W.layout(n)["rho"]][np.searchsorted(np.concatenate([[0.0], depth]), z.astype(np.float64), "right")]
+        got = got.cpu().numpy()
+        assert np.max(np.abs(got - want)) <= 2e-6 * np.max(np.abs(want))
+
+
 def test_sld_profile_sharp_steps_host_batch_and_flags():
     d = [120.0, 35.0]
     rho = [0.0, 4.1e-6, -0.4e-6, 2.07e-6]
