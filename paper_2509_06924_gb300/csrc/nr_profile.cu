@@ -63,6 +63,13 @@ __device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ 
 // finite, by the exponent bits (an FP64 comparison of a warp takes 16 cycles of its SM)
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
+// below zero, by the bits (the float of a tiny negative number is -0)
+__device__ __forceinline__ bool negative_bits(double v)
+{
+    const int h = __double2hiint(v);
+    return h < 0 && ((h & 0x7fffffff) | __double2loint(v)) != 0;
+}
+
 // One warp stages stack parameters p (n layers) into st.
 __device__ void stage_profile(ProfileStack &st, const double *p, int n, int lane, int32_t *status)
 {
@@ -108,7 +115,7 @@ __device__ void stage_profile(ProfileStack &st, const double *p, int n, int lane
             st.med[j] = make_float4((float)(ij1 - ij), reach, (float)rj1, (float)ij1);
             if (j == 0) st.rho0 = (float)rj;
             bad |= !finite_bits(depth) || !finite_bits(rj) || !finite_bits(rj1) || !finite_bits(ij) ||
-                   !finite_bits(ij1) || !finite_bits(sgd) || sg < 0.f;
+                   !finite_bits(ij1) || !finite_bits(sgd) || negative_bits(sgd);
         }
     }
     bad = __any_sync(kAll, bad);

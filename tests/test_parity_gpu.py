@@ -819,6 +819,16 @@ def test_sld_profile_runs(nz, order):
     ctx.close()
 
 
+@pytest.mark.parametrize("sigma,flagged", [(-1e-60, True), (-5e-324, True), (-3.0, True), (-0.0, False), (1e-60, False)])
+def test_sld_profile_flags_any_negative_roughness(sigma, flagged):
+    wl = custom_workload([(1, W.pack([50.0], [0.0, 4e-6, 2e-6], [0.0, 0.0], [sigma, 3.0], 1.0, 0.0), 0)],
+                         [(W.log_grid(10, 0.01, 0.2), np.zeros(10))])
+    ctx = nr.Context(n_quad=wl.n_quad)
+    ctx.sld_profile(nr.Batch.from_workload(wl), torch.linspace(-10, 90, 41, device="cuda"))
+    assert bool(ctx.device_status() & nr.NR_FLAG_NONFINITE_PARAM) == flagged
+    ctx.close()
+
+
 def test_sld_profile_sharp_steps_on_grid_depths():
     """Sharp steps whose depths, added up in FP64 from thicknesses in tenths, lie
     on float grid points take the deeper medium's value there, in stacks of more
