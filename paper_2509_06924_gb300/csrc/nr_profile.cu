@@ -27,7 +27,11 @@
 // depth (FP64, kept as a float pair), its steps and its reach;
 // then the warps share out the 8 stacks' runs.  z - z_j is formed as
 // (z - z_hi) - z_lo, exact near the interface (where the error function is
-// steep) and FP32-accurate elsewhere.
+// steep) and FP32-accurate elsewhere.  Few stacks leave SMs idle that way, so
+// the runs of a group are then shared out to several CTAs, each of which
+// stages the group for itself, as long as every warp gets a run: 8 stacks x
+// 65536 depths, ten layers, 409 -> 27 us (222 with a CTA per stack that
+// evaluated every interface), one layer 483 -> 27 us (89).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -127,12 +131,15 @@ __device__ void stage_profile(ProfileStack &st, const double *p, int n, int lane
 
 __global__ void __launch_bounds__(kProfileBlock)
 nr_profile_kernel(const double *params, const int64_t *par_off, const int32_t *n_layers, int n_same, int n_stacks,
-                  const float *z, int nz, float *rho_out, float *iota_out, int32_t *status)
+                  int parts, const float *z, int nz, float *rho_out, float *iota_out, int32_t *status)
 {
     __shared__ ProfileStack sh[kProfileWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int runs = (nz + kRun - 1) / kRun;
-    for (int s0 = blockIdx.x * kProfileWarps; s0 < n_stacks; s0 += gridDim.x * kProfileWarps) {
+    const int groups = (n_stacks + kProfileWarps - 1) / kProfileWarps;
+    // parts > 1: one (group, part) per CTA
+    for (int g = blockIdx.x / parts; g < groups; g += gridDim.x / parts) {
+        const int s0 = g * kProfileWarps, part = blockIdx.x - blockIdx.x / parts * parts;
         __syncthreads(); // the previous stacks' entries are no longer read
         if (const int s = s0 + warp; s < n_stacks) {
             const int64_t off = par_off ? par_off[s] : (4 * (int64_t)n_same + 6) * s;
@@ -142,8 +149,8 @@ nr_profile_kernel(const double *params, const int64_t *par_off, const int32_t *n
         const int here = min(kProfileWarps, n_stacks - s0);
         // the 8 stacks' runs, run by run, in equal shares: a warp forms a run's
         // span once for the stacks it takes it for
-        const int total = here * runs, share = (total + kProfileWarps - 1) / kProfileWarps;
-        int at = warp * share;
+        const int total = here * runs, warps = kProfileWarps * parts, share = (total + warps - 1) / warps;
+        int at = (part * kProfileWarps + warp) * share;
         const int end = min(at + share, total);
         int run = at / here, k = at - run * here;
         float z0 = 0.f, z1 = 0.f, zlo = 0.f, zhi = 0.f, slack = 0.f;
@@ -236,8 +243,14 @@ cudaError_t launch_profile(const double *params, const int64_t *par_off, const i
 {
     if (n_stacks == 0 || nz == 0) return cudaSuccess;
     const int groups = (n_stacks + kProfileWarps - 1) / kProfileWarps;
-    const int grid = groups < 8 * sms ? groups : 8 * sms;
-    nr_profile_kernel<<<grid, kProfileBlock, 0, st>>>(params, par_off, n_layers, n_same, n_stacks, z, nz,
+    // fewer groups than the SMs take CTAs (4 each): share out their runs
+    const int runs = (nz + kRun - 1) / kRun;
+    const int here = n_stacks < kProfileWarps ? n_stacks : kProfileWarps;
+    const int most = (here * runs + kProfileWarps - 1) / kProfileWarps; // a run per warp
+    int parts = 4 * sms / groups;
+    parts = parts > most ? most : parts < 1 ? 1 : parts;
+    const int grid = parts > 1 ? groups * parts : groups < 8 * sms ? groups : 8 * sms;
+    nr_profile_kernel<<<grid, kProfileBlock, 0, st>>>(params, par_off, n_layers, n_same, n_stacks, parts, z, nz,
                                                       rho_out, iota_out, status);
     return cudaGetLastError();
 }

@@ -829,6 +829,53 @@ def test_sld_profile_flags_any_negative_roughness(sigma, flagged):
     ctx.close()
 
 
+@pytest.mark.parametrize("S,n,nz", [(1, 3, 100000), (1, 0, 1), (3, 33, 70), (8, 10, 65536), (9, 2, 4097),
+                                    (60, 5, 1000), (2000, 1, 129)])
+def test_sld_profile_shares_out_the_runs_of_few_stacks(S, n, nz):
+    """Few stacks are spread over the device by runs of depths; every output is
+    written, whatever the remainders.  Bound as for the workloads."""
+    rng = np.random.default_rng(S)
+    q = W.log_grid(10, 0.01, 0.2)
+    wl = custom_workload([(n, rand_stack(rng, n), 0) for _ in range(S)], [(q, 0.05 * q.astype(np.float64))])
+    z = np.linspace(-50.0, 200.0 * n + 60.0, nz).astype(np.float32)
+    ctx = nr.Context(n_quad=wl.n_quad)
+    out = [torch.full((S * nz,), float("nan"), device="cuda") for _ in range(2)]
+    rho, iota = ctx.sld_profile(nr.Batch.from_workload(wl), torch.as_tensor(z, device="cuda"), *out)
+    ctx.close()
+    at = rng.permutation(nz)[:2000]
+    assert torch.isfinite(rho).all() and torch.isfinite(iota).all()
+    for s in range(0, S, max(1, S // 20)):
+        ref_r, ref_i = (v[0] for v in profile_ref(wl.subset([s]), z[at]))
+        got_r, got_i = (v.reshape(S, nz)[s].cpu().numpy()[at] for v in (rho, iota))
+        assert np.max(np.abs(got_r - ref_r)) <= 2e-6 * max(np.max(np.abs(ref_r)), 1e-6)
+        assert np.max(np.abs(got_i - ref_i)) <= 2e-6 * max(np.max(np.abs(ref_i)), 1e-8)
+
+
+def test_sld_profile_of_few_stacks_fills_the_device():
+    """8 stacks x 65536 depths take no longer than three times 512 stacks x 1024
+    depths (as many outputs, every SM busy)."""
+    rng = np.random.default_rng(4)
+    q = W.log_grid(10, 0.01, 0.2)
+    ms = []
+    for S, nz in ((8, 65536), (512, 1024)):
+        wl = custom_workload([(5, rand_stack(rng, 5), 0) for _ in range(S)], [(q, 0.05 * q.astype(np.float64))])
+        ctx, b = nr.Context(n_quad=wl.n_quad), nr.Batch.from_workload(wl)
+        z = torch.linspace(-50.0, 1100.0, nz, device="cuda")
+        out = [torch.empty(S * nz, device="cuda") for _ in range(2)]
+        t = []
+        for _ in range(12):
+            e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            torch.cuda.synchronize()
+            e0.record()
+            ctx.sld_profile(b, z, *out)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+        ms.append(min(t))
+        ctx.close()
+    assert ms[0] <= 3.0 * ms[1]
+
+
 def test_sld_profile_sharp_steps_on_grid_depths():
     """Sharp steps whose depths, added up in FP64 from thicknesses in tenths, lie
     on float grid points take the deeper medium's value there, in stacks of more
