@@ -767,7 +767,7 @@ nr_status launch_device(nr_ctx *ctx, Plan &pl, const nr_batch *b, int mode, floa
 // device status word sees the timing launches like any call.  With
 // NR_TUNE_CACHE set, a bucket whose key is in the cache file takes the
 // stored shape without timing, and new choices are appended to the file.
-constexpr int kTunerVersion = 3;
+constexpr int kTunerVersion = 4; // 4: the teams per SM that a stored shape names are the ones that run
 
 std::string tune_key(const nr_ctx *ctx, int mode, int nmax, int items)
 {

@@ -151,7 +151,7 @@ __device__ __noinline__ float roll_drain(const float2 (*q)[kEqCap], const int *q
 // ---------------------------------------------------------------- kernel --
 template <int MODE, int NMAX>
 __global__ void __launch_bounds__(RollTraits<NMAX, MODE == kGradRes>::BLOCK, 1)
-nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
+nr_roll_kernel(const KernelArgs ka, const QuadConst qc, const int workers)
 {
     constexpr bool RES = MODE == kGradRes;
     constexpr int NM = NMAX;
@@ -227,9 +227,10 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc)
     }
     const float g_max = fmaxf(fabsf(qc.g_hi[0]), fabsf(qc.g_hi[K - 1]));
 
-    // the first items go round the SMs, one team each, the rest by ticket
-    const int workers = gridDim.x * RT::TEAMS;
+    // `workers` teams take items (the launch's request; the others of the last
+    // round of CTAs stay idle): the first ones go round the SMs, the rest by ticket
     int item = team * gridDim.x + blockIdx.x;
+    if (item >= workers) item = ka.n_items;
     for (; item < ka.n_items;) {
         const WorkItem wi = ka.items[item];
         if (tid == 0) {
@@ -716,7 +717,7 @@ cudaError_t roll_launch_one(int workers, const KernelArgs &a, const QuadConst &q
     if (e != cudaSuccess) return e;
     const int full = (workers + RT::TEAMS - 1) / RT::TEAMS;
     const int grid = full > sms ? full : workers < sms ? workers : sms;
-    nr_roll_kernel<MODE, NMAX><<<grid, RT::BLOCK, RT::DYN, st>>>(a, qc);
+    nr_roll_kernel<MODE, NMAX><<<grid, RT::BLOCK, RT::DYN, st>>>(a, qc, workers);
     return cudaGetLastError();
 }
 

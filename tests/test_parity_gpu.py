@@ -597,6 +597,35 @@ def test_chunk_choice_of_small_batches(n, S, whole):
     check_bounds(sub, errs, {"loglik_g": TOL_LL, "grad": TOL_G})
 
 
+def test_requested_consumers_are_the_ones_that_run():
+    """grid_ctas counts the teams of the multi-layer gradients: one per SM leaves
+    three quarters of an SM's warps out (measured: a little over half its rate).
+    Results do not depend on it."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(12)
+    q = W.log_grid(100, 0.005, 0.25)
+    wl = custom_workload([(10, rand_stack(rng, 10), 0) for _ in range(8 * sms)], [(q, 0.04 * q.astype(np.float64))])
+    ms, res = {}, []
+    for teams in (sms, 4 * sms):
+        ctx, b = nr.Context(n_quad=wl.n_quad, grid_ctas=teams), nr.Batch.from_workload(wl)
+        assert ctx.plan_info(b)["grid_ctas"] >= 1
+        assert [g["grid"] for g in ctx.plan_groups(b, grad=True)] == [teams]
+        t = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            torch.cuda.synchronize()
+            e0.record()
+            out = ctx.loglik_grad(b)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+        ms[teams] = min(t)
+        res.append(out)
+        ctx.close()
+    assert all(torch.equal(a, b) for a, b in zip(*res))
+    assert ms[sms] >= 1.35 * ms[4 * sms]
+
+
 def test_host_memory_calls_match_device_calls():
     wl = W.make_workload("uneven", n_stacks=20)
     ctx = nr.Context(n_quad=wl.n_quad)
