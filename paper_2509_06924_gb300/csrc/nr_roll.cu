@@ -416,6 +416,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc, const int workers)
                 if (!qok.x) R.x = __int_as_float(0x7fffffff);
                 if (!qok.y) R.y = __int_as_float(0x7fffffff);
             }
+            __syncwarp(); // the wait is .aligned: lanes with a bad Q point are back
             tmem_wait_store();
 
             // a8-a10: smearing sum, model, residual, adjoint seed
@@ -595,6 +596,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc, const int workers)
             };
             // the staged sign of 1/err marks Q points whose nodes may lie below an
             // interior edge or in its band (warp-uniform choice)
+            __syncwarp(); // the sweeps begin with an .aligned load, whichever lanes stored above
             if (renorm) sweep(std::true_type{}, std::true_type{});
             else if (__any_sync(kFull, reach[0] || reach[1])) sweep(std::true_type{}, std::false_type{});
             else sweep(std::false_type{}, std::false_type{});

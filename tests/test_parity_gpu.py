@@ -523,6 +523,34 @@ def test_a_bad_q_point_leaves_the_others():
     assert np.max(np.abs(np.log(m[:, keep]) - np.log(good[:, keep]))) <= TOL_M
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 12, 24, 40])
+def test_a_bad_q_point_in_a_gradient_spoils_its_own_stacks(n):
+    """Two stacks on two curves, one with a non-positive and a NaN point: the flag
+    is raised, that stack's gradient is NaN, the other's within the bounds."""
+    rng = np.random.default_rng(20 + n)
+    q = W.log_grid(90, 0.01, 0.2)
+    wl = custom_workload([(n, rand_stack(rng, n, d_range=(20, 100)), i) for i in (0, 1)],
+                         [(q, 0.03 * q.astype(np.float64))] * 2)
+    good = wl.subset([1])
+    ref_ll, ref_g, ref_r = oracle.batch("grad_res", good.n_layers, good.params, good.dataset, good.q_off, good.q,
+                                        good.dq, good.r_obs, good.r_err, good.n_quad)
+    wl.q = wl.q.copy()
+    wl.q[[7, 40]] = (-0.01, np.nan)
+    for res in (False, True):
+        ctx = nr.Context(n_quad=wl.n_quad)
+        b = nr.Batch.from_workload(wl)
+        out = ctx.loglik_grad_res(b) if res else ctx.loglik_grad(b)
+        ll, g = (t.cpu().numpy() for t in out[:2])
+        assert ctx.device_status() & nr.NR_FLAG_BAD_Q
+        ctx.close()
+        g = g.reshape(2, -1)
+        assert np.isnan(ll[0]) and np.isnan(g[0, 4 * n + 4]) and (n < 1 or np.isnan(g[0, 0]))
+        assert abs(ll[1] - ref_ll[0]) <= TOL_LL * abs(ref_ll[0])
+        assert grad_err(good, g[1], ref_g) <= TOL_G
+        if res:
+            assert res_err(good, g[1], out[2].cpu().numpy()[1:], ref_g, ref_r) <= TOL_G
+
+
 def test_zero_resolution_is_unsmeared():
     wl = W.make_workload("thick_oxide", n_stacks=16)
     wl.dq = np.zeros_like(wl.dq)
