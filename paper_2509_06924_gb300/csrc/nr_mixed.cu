@@ -189,7 +189,7 @@ nr_mixed_kernel(const KernelArgs ka, const QuadConst qc)
         // the 1-layer bucket holds exactly-1-layer stacks: n is a constant there
         const int n = (NMAX == 1 && NR_EXACT1) ? 1 : si.n;
         const double *p = ka.params + si.par_off;
-        stage_stack<NM>(sm, &sm.nc_big[0], p, n, tid, ka.status);
+        stage_stack<NM, 0>(sm, &sm.nc_big[0], p, n, tid, ka.status);
 
         // per-thread partial gradients (FP32; reduced in FP64 per item)
         float accr[GRAD && !T::SMEM_ACC ? T::NACC : 1];

@@ -319,7 +319,9 @@ nr_pair_kernel(const KernelArgs ka, const QuadConst qc)
             first0 = fetch(wi.q_lo + tid);
             first1 = fetch(wi.q_lo + tid + BLOCK);
         }
-        stage_stack<NM>(sm, &sm.nc_big[par], p, n, tid, ka.status);
+        // one layer cannot grow (the fronting medium propagates); its log-likelihood takes no table
+        constexpr int FLAGS = NMAX == 1 ? (TAB ? kNcBig : 0) : kNcBig | kNcGrows;
+        stage_stack<NM, FLAGS>(sm, &sm.nc_big[par], p, n, tid, ka.status);
         if (QUANT && tid == 0) sm.p_max = 0;
         __syncthreads();
         if (tid == 0) sm.nc_big[par ^ 1] = 0;

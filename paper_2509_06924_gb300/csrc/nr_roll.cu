@@ -253,7 +253,7 @@ nr_roll_kernel(const KernelArgs ka, const QuadConst qc, const int workers)
         const StackInfo si = ka.stacks[wi.stack];
         const int n = si.n;
         const double *p = ka.params + si.par_off;
-        stage_stack<NM>(sm, &sm.nc_big[0], p, n, tid, ka.status);
+        stage_stack<NM, kNcBig | kNcGrows>(sm, &sm.nc_big[0], p, n, tid, ka.status);
         for (int i = lane; i < (n + 2) * 32; i += 32) acc[i] = 0.f;
 
         // step j's four sums: over the quad's lanes, one sum left in each lane
