@@ -24,7 +24,7 @@ INCLUDE = os.path.join(ROOT, "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["nr_mixed.cu", "nr_pair.cu", "nr_roll.cu", "nr_fp64.cu", "nr_noalloc.cu", "nr_profile.cu", "nr_hmc.cu", "nr_vi.cu"]
 CPP_SOURCES = ["nr_api.cpp", "nr_tune.cpp"]
-HEADERS = ["nr_internal.h", "nr_device.cuh", "nr_pair.cuh", "nr_cofit.cuh"]
+HEADERS = ["nr_internal.h", "nr_once.h", "nr_device.cuh", "nr_pair.cuh", "nr_cofit.cuh"]
 
 
 def _cuda_home() -> str:

@@ -39,6 +39,7 @@
 
 #include "nr_device.cuh"
 #include "nr_internal.h"
+#include "nr_once.h"
 
 namespace nrimpl {
 namespace {
@@ -785,11 +786,12 @@ template <int MODE, int NMAX, int KC>
 cudaError_t launch_k(int grid, const KernelArgs &a, const QuadConst &qc, cudaStream_t st)
 {
     using T = Traits<MODE, NMAX>;
-    static bool attr_done = false; // per process: the attribute belongs to the function
-    if (!attr_done) {
-        cudaError_t e = set_smem_attr<MODE, NMAX, KC>();
+    if constexpr (T::DYN > 0) {
+        static OncePerDevice attr;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = attr.run(dev, set_smem_attr<MODE, NMAX, KC>);
         if (e != cudaSuccess) return e;
-        attr_done = true;
     }
     nr_mixed_kernel<MODE, NMAX, KC><<<grid, T::BLOCK, T::DYN, st>>>(a, qc);
     return cudaGetLastError();

@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "nr_internal.h"
+#include "nr_once.h"
 #include "nr_pair.cuh"
 
 namespace nrimpl {
@@ -707,14 +708,10 @@ template <int MODE, int NMAX>
 cudaError_t roll_launch_one(int workers, const KernelArgs &a, const QuadConst &qc, cudaStream_t st)
 {
     using RT = RollTraits<NMAX, MODE == kGradRes>;
-    static bool attr_done = false; // per process: the attribute belongs to the function
-    if (!attr_done) {
-        const cudaError_t e = roll_attr<MODE, NMAX>();
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static OncePerDevice attr;
     int dev = 0, sms = 1;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = attr.run(dev, roll_attr<MODE, NMAX>);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int full = (workers + RT::TEAMS - 1) / RT::TEAMS;

@@ -259,3 +259,42 @@ def test_cost_partition_covers_every_stack_once_and_balances():
         # LPT greedy: the largest load is within the largest single cost of the mean
         assert loads.max() <= loads.mean() + cost.max() + 1e-9
         assert all(np.all(np.diff(p) > 0) for p in parts)
+
+
+def test_kernel_attributes_are_set_on_every_device(tmp_path):
+    """A kernel's opt-in to large dynamic shared memory belongs to one device:
+    every device sets it, once, again after a failure, from any thread.  (Where
+    a process holds contexts on several GPUs; here a fake device counts.)"""
+    import subprocess
+    src = tmp_path / "once.cpp"
+    src.write_text("""
+        #include "nr_once.h"
+        #include <cstdio>
+        #include <thread>
+        #include <vector>
+        int main()
+        {
+            static nrimpl::OncePerDevice once;
+            std::atomic<int> calls[70] = {};
+            int fail = 1; // the first attempt on device 3 fails
+            auto on = [&](int d) { return once.run(d, [&] { ++calls[d]; return d == 3 ? fail : 0; }); };
+            if (on(3) != 1) return 1;
+            fail = 0;
+            for (int r = 0; r < 3; ++r)
+                for (int d : {0, 1, 3, 63, 64})
+                    if (on(d) != 0) return 2;
+            const bool ok = calls[0] == 1 && calls[1] == 1 && calls[3] == 2 && calls[63] == 1 && calls[64] == 3;
+            std::vector<std::thread> t; // device 7 from many threads: set before any of them goes on
+            std::atomic<int> early{0};
+            for (int i = 0; i < 16; ++i) t.emplace_back([&] { if (on(7) != 0 || calls[7] == 0) ++early; });
+            for (auto &x : t) x.join();
+            return ok && early == 0 ? 0 : 3;
+        }""")
+    exe = tmp_path / "once"
+    csrc = os.path.join(os.path.dirname(nr.__file__), "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", csrc, str(src), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0
+    for name in ("nr_roll.cu", "nr_mixed.cu"):  # and the launchers use it
+        with open(os.path.join(csrc, name)) as f:
+            text = f.read()
+        assert "OncePerDevice" in text and "attr_done" not in text
