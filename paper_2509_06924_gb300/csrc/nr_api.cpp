@@ -364,7 +364,7 @@ std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std:
     // the stacks of a group by kind (layers and points): a batch has few
     struct Kind {
         int n;
-        int64_t len;
+        int32_t tiles; // of the whole dataset
         double count;
     };
     std::vector<std::vector<Kind>> kinds(gs.size());
@@ -372,14 +372,13 @@ std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std:
         const GroupSpan &g = gs[k];
         const ItemCost ic = item_cost(mode, g.nmax);
         ChunkCand c{chunk, 0.0, 0.0, 0};
+        // a chunk is whole tiles, or the whole dataset: a stack's tiles stay the same
+        const int32_t t = (int32_t)std::min<int64_t>((chunk + g.tile_q - 1) / g.tile_q, INT32_MAX);
         for (const Kind &kd : kinds[k]) {
-            const int64_t len = std::max<int64_t>(kd.len, 1), ch = std::min(chunk, len);
-            const int64_t nch = (len + ch - 1) / ch, rest = len - (nch - 1) * ch;
-            const double w = ic.tile * (kd.n + 1.0);
-            const int64_t t = (ch + g.tile_q - 1) / g.tile_q, tr = (rest + g.tile_q - 1) / g.tile_q;
-            c.total += kd.count * (w * (double)((nch - 1) * t + tr) + (double)nch * ic.item);
-            c.big = std::max(c.big, w * (double)t + ic.item);
-            c.items += (int64_t)kd.count * nch;
+            const double w = ic.tile * (kd.n + 1.0), items = kd.tiles <= t ? 1 : (kd.tiles + t - 1) / t;
+            c.total += kd.count * (w * kd.tiles + items * ic.item);
+            c.big = std::max(c.big, w * std::min(t, kd.tiles) + ic.item);
+            c.items += (int64_t)(kd.count * items);
         }
         return c;
     };
@@ -391,13 +390,16 @@ std::vector<int64_t> choose_chunks(const Plan &pl, int mode, int sms, const std:
         for (size_t i = gs[k].i0; i < gs[k].i1; ++i) whole[k] = std::max(whole[k], dlen(order[i]));
     }
     if (nst >= kChunkWaves * most) return whole;
+    auto tiles_of = [](int64_t len, int tile_q) {
+        return (int32_t)std::min<int64_t>((std::max<int64_t>(len, 1) + tile_q - 1) / tile_q, INT32_MAX / 2);
+    };
     for (size_t k = 0; k < gs.size(); ++k) {
         std::unordered_map<int64_t, size_t> at;
         for (size_t i = gs[k].i0; i < gs[k].i1; ++i) {
             const int s = order[i];
             const int64_t len = dlen(s);
             const auto found = at.try_emplace(len * (NR_MAX_LAYERS + 1) + pl.n_layers[s], kinds[k].size());
-            if (found.second) kinds[k].push_back(Kind{pl.n_layers[s], len, 0.0});
+            if (found.second) kinds[k].push_back(Kind{pl.n_layers[s], tiles_of(len, gs[k].tile_q), 0.0});
             kinds[k][found.first->second].count += 1.0;
         }
         const ChunkCand w = cost_of(k, whole[k]);
