@@ -531,11 +531,13 @@ def _autograd_function():
             n_layers, n_stacks = ctx_.layout
             # stacks of one layer count: one broadcast product (the general
             # form copies the counts to the device and waits for it twice:
-            # 477 -> 338 us a step of a one-curve fit, forward included)
+            # 477 -> 338 us a step of a one-curve fit, forward included); both
+            # refuse a gradient of another length than the stacks' packed one
             if n_stacks and (n_layers == n_layers[0]).all():
-                return (g.view(n_stacks, -1) * grad_ll.unsqueeze(1)).reshape(-1), None, None
-            per = torch.as_tensor(4 * n_layers.astype(np.int64) + 6, device=g.device)
-            scale = torch.repeat_interleave(grad_ll, per, output_size=g.numel())
+                rows = g.view(n_stacks, 4 * int(n_layers[0]) + 6)
+                return (rows * grad_ll.unsqueeze(1)).reshape(-1), None, None
+            per = 4 * n_layers.astype(np.int64) + 6
+            scale = torch.repeat_interleave(grad_ll, torch.as_tensor(per, device=g.device), output_size=int(per.sum()))
             return g * scale, None, None
 
     return NRLogLik

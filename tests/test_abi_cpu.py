@@ -298,3 +298,30 @@ def test_kernel_attributes_are_set_on_every_device(tmp_path):
         with open(os.path.join(csrc, name)) as f:
             text = f.read()
         assert "OncePerDevice" in text and "attr_done" not in text
+
+
+@pytest.mark.parametrize("n_layers", [[1, 1], [1, 2], [0], [3]])
+def test_autograd_backward_refuses_a_wrong_length(n_layers):
+    """A parameter buffer longer than the packed stacks is refused by backward
+    (weights must not land on other stacks' entries); one of the right length
+    takes each stack's own weight.  The device call is replaced by numbers."""
+    torch = pytest.importorskip("torch")
+    n = np.array(n_layers, np.int32)
+    per = 4 * n.astype(np.int64) + 6
+
+    class Fake:
+        def loglik_grad(self, batch):
+            return torch.zeros(n.size, dtype=torch.float64), torch.arange(batch.params.numel(), dtype=torch.float64)
+
+    w = torch.linspace(2.0, 3.0, n.size, dtype=torch.float64)
+    for extra in (0, 4, 2 * n.size):
+        params = torch.zeros(int(per.sum()) + extra, dtype=torch.float64, requires_grad=True)
+        batch = nr.Batch(n, np.zeros(n.size, np.int32), np.array([0, 1]), params, None, None)
+        ll = nr.loglik_autograd(params, Fake(), batch)
+        if extra:
+            with pytest.raises(RuntimeError):
+                torch.autograd.grad(ll, params, grad_outputs=w)
+        else:
+            (g,) = torch.autograd.grad(ll, params, grad_outputs=w)
+            want = torch.arange(params.numel(), dtype=torch.float64) * torch.repeat_interleave(w, torch.as_tensor(per))
+            assert torch.equal(g, want)
