@@ -164,6 +164,22 @@ def test_flop_table_is_monotone_and_positive():
     assert all(bench.flops_per_eval_fwd(n, 21) < bench.flops_per_eval(n, 21) for n in range(0, 21))
 
 
+def test_roofline_counts_what_the_kernels_execute():
+    """The roofline's flops per evaluation are the ones that the committed ncu
+    summaries count, less what is left out of the count (reductions, idle slots
+    of a tile, the tiles near or below an interior edge): 0 to 10 %."""
+    import bench
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for name, count in (("nr_grad_thick_oxide", bench.executed_flops(1, 21)),
+                        ("nr_grad_vi_step", bench.executed_flops(12, 21)),
+                        ("nr_pair_loglik_thick_oxide", bench.executed_flops_fwd(1, 21))):
+        with open(os.path.join(root, "profiles", name + ".txt")) as f:
+            executed = float(re.search(r"fp32 flops per eval: ([\d.]+)", f.read()).group(1))
+        assert 0.9 * executed <= count <= executed
+    f = [bench.executed_flops(n, 21) for n in range(65)]
+    assert all(b > a for a, b in zip(f, f[1:])) and all(x < bench.flops_per_eval(n, 21) for n, x in enumerate(f) if n)
+
+
 def test_peak_probe_library_builds_and_exports():
     from paper_2509_06924_gb300 import _build
     lib = ctypes.CDLL(_build.build_peak())
