@@ -416,8 +416,9 @@ __device__ __forceinline__ void k0_square(float k0h, float k0l, float &p_hi, flo
 }
 
 // One queued interior-edge evaluation: the entry keeps the node k_0 (hi, lo),
-// Z and Xbar_{j-1}; k_{j-1}, k_j and k_{j+1} are formed again from the node
-// exactly as the sweeps form them.
+// Z and Xbar_{j-1}; k_{j-1}, k_j and k_{j+1} are formed again from the node (in
+// their last roundings they may differ from the sweep's, which may split the
+// squares by a common quantum and keep another part of the root's refinement).
 __device__ __forceinline__ float2 edge_entry_ubar(float2 node, float2 Z, float2 Xbu, int j, int n,
                                                   const float4 *med, const float *sig, const float4 *adj)
 {

@@ -17,9 +17,9 @@
 // from a polynomial where the stack's roughnesses allow it, and layer phases
 // are staged in table steps.  Against the Moebius form with table phases, the
 // later changes below included: 16384 one-layer stacks x 400 Q x 21 nodes,
-// gradient 1.464 -> 1.292 ms, log-likelihood 0.820 -> 0.749 ms; 12288
-// ten-layer stacks, model curves 1.779 -> 1.426 ms; 10000 stacks of 1-20
-// layers, log-likelihood 1.623 -> 1.407 ms.
+// gradient 1.464 -> 1.310 ms, log-likelihood 0.820 -> 0.756 ms; 12288
+// ten-layer stacks, model curves 1.779 -> 1.446 ms; 10000 stacks of 1-20
+// layers, log-likelihood 1.623 -> 1.381 ms.
 //
 // The forward modes run the same code up to the smearing sum (model: write
 // scale S + bkg; log-likelihood: the residual terms) and no adjoint.

@@ -20,8 +20,8 @@
 // and only the interfaces that a ballot names are evaluated, each as its
 // difference from what the base already counts.  That holds for any order of
 // the depths (a run then just spans more).  16384 stacks of ten layers x 512
-// depths, both curves: 165 -> 45 us a call (1.6 TB/s of its 67 MB output and
-// parameters; stacks of one layer count upload no metadata either).
+// depths, both curves: 165 -> 49 us a call (1.5 TB/s of its 67 MB output and
+// 6 MB of parameters; stacks of one layer count upload no metadata either).
 //
 // A CTA stages 8 stacks at a time, one per warp: lane j forms interface j's
 // depth (FP64, kept as a float pair), its steps and its reach;

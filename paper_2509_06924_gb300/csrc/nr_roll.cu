@@ -11,10 +11,10 @@
 // the cheapest, is formed again.  The recursion runs in projective form
 // (nr_pair.cuh), without divisions and with short chains in both directions.
 // Against forming the factors twice in the Moebius form, with everything in
-// shared memory: 196608 twelve-layer stacks x 300 Q x 21 nodes 150.8 -> 101.0
-// ms, 12288 ten-layer stacks (150-300 Q, 17 nodes) 5.03 -> 3.35 ms, 10000
-// stacks of 1-20 layers 5.83 -> 3.72 ms; 1024 stacks of 21-64 layers, which
-// ran one evaluation per thread, 3.69 -> 1.62 ms.  Storing 32 bytes a layer
+// shared memory: 196608 twelve-layer stacks x 300 Q x 21 nodes 150.8 -> 104.5
+// ms, 12288 ten-layer stacks (150-300 Q, 17 nodes) 5.03 -> 3.50 ms, 10000
+// stacks of 1-20 layers 5.83 -> 3.96 ms; 1024 stacks of 21-64 layers, which
+// ran one evaluation per thread, 3.69 -> 1.74 ms.  Storing 32 bytes a layer
 // in TMEM and reading them back costs about 30 cycles per warp and layer (16
 // warps an SM), forming them again 200.
 //

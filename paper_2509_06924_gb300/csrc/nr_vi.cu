@@ -24,7 +24,7 @@
 // and theta is formed once per parameter, not once per packed slot.  100
 // restarts of a 51-parameter co-fit: sample 24, gather 6, pull-back 16 and
 // Adam 14 us as four launches of a warp per restart; the iteration fell from
-// 193 to 172 us (165 with the present gradient kernel).
+// 193 to 172 us (176 with the present gradient kernel).
 #include <cuda_runtime.h>
 
 #include <cmath>
